@@ -32,7 +32,9 @@ struct dkv_plan {
     int32_t* d_idx = nullptr;   // [kept]
     int32_t* d_status = nullptr;
     float* d_work = nullptr;    // split-K partials
-    int32_t* d_slab_count = nullptr;  // [B*H_kv][cols][2] arrival / written counters of the fused combine
+    float* d_exch = nullptr;    // exchange of the fused merge: slots x kMaxCols x (128 + 2) words, 0 between launches
+    int64_t exch_slots = 0;     // (CTA, slab) slots of the exchange
+    int32_t* d_slab_count = nullptr;  // [B*H_kv][cols][2] arrival / done counters of the tcgen05 kernel's merge
     dkv::DecodeConfig cfg{};         // the decode step's kernel (cfg_f32 or cfg_mma)
     dkv::DecodeConfig cfg_f32{};     // fp32 kernel (caches of 2^31 rows or more)
     dkv::DecodeConfig cfg_mma{};     // tensor-core kernel of the decode step
@@ -166,9 +168,9 @@ dkv_status plan_configs(dkv_plan* p)
     cudaGetDevice(&p->device);
     cudaError_t e;
     if ((e = dkv::decode_config(p->G, p->B, &p->cfg_f32)) != cudaSuccess) return cuda_fail(e, "decode_config");
-    if ((e = dkv::decode_config_mma(p->G, p->B, 0, &p->cfg_mma)) != cudaSuccess ||
-        (e = dkv::decode_config_mma(p->G, p->B, 1, &p->cfg_multi1)) != cudaSuccess ||
-        (e = dkv::decode_config_mma(p->G, p->B, 2, &p->cfg_multi)) != cudaSuccess)
+    if ((e = dkv::decode_config_mma(p->G, p->B, p->s.H_kv, 0, &p->cfg_mma)) != cudaSuccess ||
+        (e = dkv::decode_config_mma(p->G, p->B, p->s.H_kv, 1, &p->cfg_multi1)) != cudaSuccess ||
+        (e = dkv::decode_config_mma(p->G, p->B, p->s.H_kv, 2, &p->cfg_multi)) != cudaSuccess)
         return cuda_fail(e, "decode_config (tensor cores)");
     if ((e = dkv::decode_config_tc(p->G, p->B, &p->cfg_tc)) != cudaSuccess) return cuda_fail(e, "decode_config (tcgen05)");
     // Warp records: the mma.sync and fp32 kernels (up to kMaxCols columns); CTA
@@ -181,8 +183,12 @@ dkv_status plan_configs(dkv_plan* p)
     p->cols_cap = dkv::kMaxCols;
     const int64_t NHl = (int64_t)p->B * p->s.H_kv;
     p->work = dkv::workspace_layout(ctas + NHl, dkv::kTcMaxCols, warp_records, dkv::kMaxCols);
+    p->exch_slots = ctas + NHl;
     return DKV_OK;
 }
+
+// Floats of the fused merge's exchange.
+int64_t exch_floats(const dkv_plan* p) { return p->exch_slots * dkv::kMaxCols * (dkv::kHeadDim + 2); }
 
 // Places the counters (status word, then the fused combine's slab counters) as
 // one int32 block that a single memset zeroes, and the split-K workspace.
@@ -344,6 +350,7 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     ma.stride = inplace_stride;
     ma.status = p->d_status;
     if ((st = launched(dkv::launch_map(ma, stream), "map kernels")) != DKV_OK) return bail(st);
+    if ((st = plan_configs(p)) != DKV_OK) return bail(st);  // host work, while the kernels run
     // The one synchronisation: the totals (rows, kept rows, longest slab, rows of each layer).
     std::vector<int64_t> tail((size_t)3 + s->L);
     if ((e = cudaMemcpyAsync(tail.data(), ma.tail, sizeof(int64_t) * tail.size(), cudaMemcpyDeviceToHost, stream)) !=
@@ -353,14 +360,17 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     p->total_rows = tail[0];
     p->kept_rows = tail[1];
     p->layer_rows.assign(tail.begin() + 3, tail.end());
-    if ((st = plan_configs(p)) != DKV_OK) return bail(st);
     ArenaLayout lay2;
-    const size_t o_idx = lay2.take<int32_t>((size_t)p->kept_rows), o_work = lay2.take<float>((size_t)p->work.total);
+    const size_t o_idx = lay2.take<int32_t>((size_t)p->kept_rows), o_work = lay2.take<float>((size_t)p->work.total),
+                 o_exch = lay2.take<float>((size_t)exch_floats(p));
     if ((st = dalloc(reinterpret_cast<unsigned char**>(&p->d_arena2), lay2.bytes, "index list and workspace")) !=
         DKV_OK)
         return bail(st);
     p->d_idx = at<int32_t>(p->d_arena2, o_idx);
     p->d_work = at<float>(p->d_arena2, o_work);
+    p->d_exch = at<float>(p->d_arena2, o_exch);
+    if ((e = cudaMemsetAsync(p->d_exch, 0, (size_t)exch_floats(p) * sizeof(float), stream)) != cudaSuccess)
+        return bail(cuda_fail(e, "clear exchange"));
     ma.idx = p->d_idx;
     if ((st = launched(dkv::launch_map_write(ma, (int)tail[2], stream), "map write kernel")) != DKV_OK)
         return bail(st);
@@ -437,16 +447,18 @@ dkv_status dkv_plan_dense(const int32_t* ctx_len_host, int32_t B, const dkv_shap
     const size_t o_len = lay.take<int32_t>((size_t)NH), o_off = lay.take<int64_t>((size_t)NH + 1),
                  o_ioff = lay.take<int64_t>((size_t)NH + 1);
     const ZeroBlock zb = take_zeroed(lay, p, 0);
-    const size_t o_work = lay.take<float>((size_t)p->work.total);
+    const size_t o_work = lay.take<float>((size_t)p->work.total), o_exch = lay.take<float>((size_t)exch_floats(p));
     if ((st = dalloc(reinterpret_cast<unsigned char**>(&p->d_arena), lay.bytes, "plan metadata")) != DKV_OK)
         return bail(st);
     p->d_len = at<int32_t>(p->d_arena, o_len);
     p->d_off = at<int64_t>(p->d_arena, o_off);
     p->d_ioff = at<int64_t>(p->d_arena, o_ioff);
     p->d_work = at<float>(p->d_arena, o_work);
+    p->d_exch = at<float>(p->d_arena, o_exch);
     place_zeroed(p, zb);
     cudaError_t e;
     if ((e = cudaMemsetAsync(p->d_status, 0, zb.count * sizeof(int32_t), stream)) != cudaSuccess ||
+        (e = cudaMemsetAsync(p->d_exch, 0, (size_t)exch_floats(p) * sizeof(float), stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(p->d_len, len.data(), (size_t)NH * 4, cudaMemcpyHostToDevice, stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(p->d_off, off.data(), (size_t)(NH + 1) * 8, cudaMemcpyHostToDevice, stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(p->d_ioff, ioff.data(), (size_t)(NH + 1) * 8, cudaMemcpyHostToDevice, stream)) != cudaSuccess ||
@@ -613,6 +625,8 @@ dkv_status decode_args(const dkv_plan* p, int32_t layer, const void* q, const vo
     a->warp_ml = p->d_work + p->work.warp_ml;
     if (!aligned16(a->work_o) || !aligned16(a->work_ml) || !aligned16(a->warp_o) || !aligned16(a->warp_ml))
         return fail(DKV_ERR_INVALID_ARG, "split-K workspace regions are not 16-byte aligned");
+    a->exch_o = p->d_exch;
+    a->exch_ml = p->d_exch + p->exch_slots * dkv::kMaxCols * dkv::kHeadDim;
     a->out = out;
     a->slab_count = p->d_slab_count;
     a->merge_extra = fault("merge") ? 1 : 0;
@@ -681,7 +695,7 @@ dkv_status dkv_decode_multi(const dkv_plan* p, int32_t layer, const void* q, int
         // tcgen05 kernel (accumulators in TMEM).
         a.nctas = p->cfg_tc.nctas;
         dkv::CacheMaps maps;
-        const cudaError_t e = dkv::make_cache_maps(a.Kc, a.Vc, p->total_rows, &maps, fault("copy"), 16);
+        const cudaError_t e = dkv::make_cache_maps(a.Kc, a.Vc, p->total_rows, &maps, fault("copy"), 16, false);
         if (e != cudaSuccess) return cuda_fail(e, "tensor maps of the packed caches");
         st = launched(dkv::launch_decode_tc(a, maps, p->cfg_tc, stream), "multi-query decode kernel (tcgen05)");
         return st == DKV_OK ? ok() : st;

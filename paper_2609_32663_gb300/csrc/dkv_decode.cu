@@ -108,13 +108,14 @@ struct PK {
     static constexpr int kRingBytes = NW * NS * kStageBytes;
     static constexpr int kScratchBytes = NW * kWarpScratch;
     static constexpr int kBarBytes = NW * NS * 8;
-    static constexpr int kMetaBytes = NW * 6 * 4 + 16;  // first/last slab of each warp, their row bounds
+    static constexpr int kMetaBytes = TailMeta<NW>::kWords * 4;
     static constexpr int kFixedBytes = kRingBytes + kScratchBytes + kBarBytes + kMetaBytes;
     static constexpr int kStateFloats = G * (kHeadDim + 2);
     static int bytes(int B) { return kFixedBytes + seq_table_bytes(B); }
     static_assert(kFixedBytes + seq_table_bytes(kMaxB) <= 227 * 1024, "fits the opt-in shared memory of one CTA");
     static_assert(TR % RPS == 0 && 32 % TR == 0, "tile geometry");
-    static_assert(kStateFloats * 4 <= NS * kStageBytes, "a warp's final state fits in its ring");
+    static constexpr int kDepOff = (kStateFloats * 4 + 15) / 16 * 16;  // after a warp's final state
+    static_assert(kDepOff + 528 <= NS * kStageBytes, "a warp's final state and a deposit fit in its ring");
 };
 
 // Per-warp running state of one slab segment.
@@ -320,16 +321,14 @@ __device__ __forceinline__ void finish_state(State<C>& S, float (&l_all)[C::G])
 }
 
 template <class C, bool FUSED>
-__global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const DecodeArgs a)
+__global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const __grid_constant__ DecodeArgs a)
 {
     constexpr int G = C::G, LPR = C::LPR, TR = C::TR, NS = C::NS, NW = C::NW;
     constexpr int DPL = C::DPL, NCH = C::NCH, NSUM = C::NSUM;
     extern __shared__ __align__(128) unsigned char smem[];
     const SeqTable tab = seq_table_at(smem + C::kFixedBytes, a);
-    int32_t* seg_first = reinterpret_cast<int32_t*>(smem + C::kRingBytes + C::kScratchBytes + C::kBarBytes);
-    int32_t* seg_last = seg_first + NW;
-    int32_t* seg_p0 = seg_first + 2 * NW;  // [2 NW] layer rows [p0, p1) of entry 2 w (first) / 2 w + 1 (last)
-    int32_t* seg_p1 = seg_first + 4 * NW;
+    using TM = TailMeta<NW>;
+    int32_t* meta = reinterpret_cast<int32_t*>(smem + C::kRingBytes + C::kScratchBytes + C::kBarBytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sl = lane % LPR;
@@ -344,10 +343,13 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const Dec
     if (lane == 0) {
         for (int s = 0; s < NS; ++s) mbar_init(smem_u32(&my_bars[s]), 1);
         fence_proxy_async_smem();
-        seg_first[warp] = -1;
-        seg_last[warp] = -1;
+        meta[TM::kFirst + warp] = -1;
+        meta[TM::kLast + warp] = -1;
+        if (warp == 0) meta[TM::kDead] = 0;
     }
     __syncthreads();  // table, barriers and slab entries are ready
+    finish_slab_cache(a, tab, NW * 32);
+    __syncthreads();
     pdl_launch_dependents();
 
     const int R = slab_start(a, tab, NHl);
@@ -360,11 +362,14 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const Dec
                 for (int j = 0; j < G; ++j)
                     write_out<G>(a, h / a.Hkv, h % a.Hkv, j, make_float4(0.f, 0.f, 0.f, 0.f), 0.f, lane);
     }
-    const int A = part_start(c, R, a.nctas), Bc = part_start(c + 1, R, a.nctas);
+    const int P = live_parts(R, a.nctas);  // CTAs with rows
+    const int A = c < P ? part_start(c, R, P) : R, Bc = c < P ? part_start(c + 1, R, P) : R;
     if (A >= Bc) return;  // uniform: this CTA has no rows
     const int wA = A + (int)(((int64_t)(Bc - A) * warp) / NW);
     const int wB = A + (int)(((int64_t)(Bc - A) * (warp + 1)) / NW);
     unsigned char* my_ring = smem + warp * NS * C::kStageBytes;
+    if (FUSED && warp == NW - 1)  // for the end of the pass
+        meta[TM::kC0] = part_of(slab_start(a, tab, slab_containing(a, tab, NHl, A)), R, P);
     State<C> S;
     float l_all[G];
     bool have_last = false;  // S holds the state of this warp's last slab
@@ -510,17 +515,17 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const Dec
             if (h == hlast) {
                 have_last = true;  // merged with the other warps at the end
                 if (lane == 0) {
-                    seg_last[warp] = h;
-                    seg_p0[2 * warp + 1] = p0h;
-                    seg_p1[2 * warp + 1] = p1h;
+                    meta[TM::kLast + warp] = h;
+                    meta[TM::kP0 + 2 * warp + 1] = p0h;
+                    meta[TM::kP1 + 2 * warp + 1] = p1h;
                 }
             } else if (h == hfirst) {
                 const int64_t rec = (int64_t)c * NW + warp;  // this slab continues in an earlier warp
                 store_state<C>(S, l_all, a.warp_o + rec * G * kHeadDim, a.warp_ml + rec * G * 2, lane);
                 if (lane == 0) {
-                    seg_first[warp] = h;
-                    seg_p0[2 * warp] = p0h;
-                    seg_p1[2 * warp] = p1h;
+                    meta[TM::kFirst + warp] = h;
+                    meta[TM::kP0 + 2 * warp] = p0h;
+                    meta[TM::kP1 + 2 * warp] = p1h;
                 }
             } else if (FUSED) {
                 write_out_state<C>(a, S, l_all, b, g, lane);  // the whole slab lies in this warp's range
@@ -532,7 +537,8 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const Dec
 
         if (dead) {
             // After a timeout, wait (with the same bound) for the copies still in flight.
-            if (lane == 0)
+            if (lane == 0) {
+                meta[TM::kDead] = 1;
                 for (int k = 0; k < inflight; ++k) {
                     mbar_wait(smem_u32(&my_bars[stage]), phase);
                     if (++stage == NS) {
@@ -540,6 +546,7 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const Dec
                         phase ^= 1u;
                     }
                 }
+            }
         }
     }
     // The warp's own ring is idle now (every tile it issued was consumed): its
@@ -550,8 +557,11 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const Dec
                        lane);
     __syncthreads();
     pdl_wait();  // the merges write the workspace and out: the previous kernel must be done with them
-
-    cta_tail<G, NW, FUSED, G>(a, smem, NS * C::kStageBytes, seg_first, c, R, warp, lane);
+    if (FUSED && meta[TM::kDead]) {
+        dead_tail<NW>(a, tab, G, c, A, Bc, R, P, warp, lane);
+        return;
+    }
+    cta_tail<G, NW, FUSED, G>(a, smem, NS * C::kStageBytes, C::kDepOff, meta, c, A, Bc, warp, lane);
 }
 
 // ------------------------------------------------------------ combine kernel
@@ -561,10 +571,10 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const Dec
 constexpr int kCombineWarps = 8;
 constexpr int kCombineStride = kHeadDim + 4;  // floats per warp share: o[128], L, pad (16-byte rows)
 
-__global__ void __launch_bounds__(kCombineWarps * 32) decode_combine_kernel(const DecodeArgs a)
+__global__ void __launch_bounds__(kCombineWarps * 32) decode_combine_kernel(const __grid_constant__ DecodeArgs a)
 {
     extern __shared__ int32_t csmem[];
-    SeqTable tab{csmem, csmem + a.B};
+    SeqTable tab{csmem, csmem + a.B, nullptr, nullptr};
     // [kCombineWarps][kCombineStride] floats after the table, at a 16-byte boundary.
     float* red = reinterpret_cast<float*>(csmem + (((2 * a.B + 1) + 3) & ~3));
     __shared__ float wmax[kCombineWarps];
@@ -586,12 +596,11 @@ __global__ void __launch_bounds__(kCombineWarps * 32) decode_combine_kernel(cons
         if (warp == 0) outp[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
     }
-    const int P = a.nctas;
+    const int P = live_parts(R, a.nctas);
     const int c0 = part_of(p0, R, P), c1 = part_of(p1 - 1, R, P);
     float M = -INFINITY;
     for (int c = c0 + (int)threadIdx.x; c <= c1; c += kCombineWarps * 32)
-        if (part_start(c, R, P) < part_start(c + 1, R, P))
-            M = fmaxf(M, a.work_ml[(((int64_t)c + h) * a.G + j) * 2]);
+        M = fmaxf(M, a.work_ml[(((int64_t)c + h) * a.G + j) * 2]);
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, o));
     if (lane == 0) wmax[warp] = M;
@@ -603,7 +612,6 @@ __global__ void __launch_bounds__(kCombineWarps * 32) decode_combine_kernel(cons
     float Lw = 0.f;
 #pragma unroll 4
     for (int c = c0 + warp; c <= c1; c += kCombineWarps) {
-        if (part_start(c, R, P) == part_start(c + 1, R, P)) continue;
         const int64_t sj = ((int64_t)c + h) * a.G + j;
         const float2 ml = *reinterpret_cast<const float2*>(a.work_ml + sj * 2);
         const float f = (ml.x == -INFINITY) ? 0.f : ex2(ml.x - M);

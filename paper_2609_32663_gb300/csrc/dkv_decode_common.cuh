@@ -2,8 +2,8 @@
 // programmatic-dependent-launch wrappers (the mbarrier and bulk-copy ones are in
 // dkv_ptx.cuh), the per-call slab table, the stream-K row partition over the slabs of one layer, the tile cursor of a
 // warp, and the end of a CTA's pass: merging the warp states that share a slab
-// and the fused cross-CTA merge (the last CTA to finish a (slab, head) merges
-// every CTA's partial of it).
+// and the fused cross-CTA merge (the last CTA of a slab merges every CTA's
+// partial of it).
 #pragma once
 
 #include "dkv_internal.cuh"
@@ -18,6 +18,12 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxB = 512;
 constexpr float kSlack = 8.f;        // lazy-rescale threshold of the online softmax (log2 units)
 constexpr int PRE = 1;               // tiles a warp fetches before waiting for the previous kernel
+
+// A value that is the same in every lane, read from lane 0. The compiler then
+// knows it is uniform over the warp: loops and branches on it are plain ones (the
+// warp-wide votes and shuffles inside need no check for a split warp), and the
+// scalar work on it runs once a warp, in uniform registers.
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(kFull, x, 0); }
 
 // Programmatic dependent launch: let the next kernel in the stream start its
 // prologue, and wait for the previous kernel's results before reading them.
@@ -37,45 +43,72 @@ __device__ __forceinline__ void pdl_wait()
 // e_b = NA[b] + (this call appends to b ? 1 : 0). Layer rows fit in int32.
 //
 // When the layer has fewer than kSlabCache slabs, the table also holds the
-// slabs' row prefix IO[h] = ioff[h] - ioff[0] ([NHl+1]) and cache offsets
-// OFF[h] = off[h] ([NHl]), so that finding a warp's rows and streaming them
-// reads no plan metadata from global memory: a CTA that starts after the
+// slabs' first layer rows P0[h] ([NHl+1], the extra rows included) and cache
+// offsets OFF[h] = off[h] ([NHl]), so that finding a warp's rows and streaming
+// them reads no plan metadata from global memory: a CTA that starts after the
 // previous kernel has drained (the last ones to get an SM) would otherwise pay
 // a chain of dependent L2 round trips, under full HBM load, before its first
-// copy. IO and OFF are null for larger layers (read from global memory then).
+// copy. P0 and OFF are null for larger layers (computed from global memory then).
 constexpr int kSlabCache = 1024;
 struct SeqTable {
     int32_t* NA;   // [B]
     int32_t* NP;   // [B+1]
-    int32_t* IO;   // [NHl+1] or null
+    int32_t* P0;   // [NHl+1] or null
     int64_t* OFF;  // [NHl] or null
 };
 
-// Bytes of the table at an 8-byte aligned base: OFF, IO, NA, NP.
-__host__ __device__ constexpr int seq_table_bytes(int B) { return kSlabCache * 8 + kSlabCache * 4 + (2 * B + 1) * 4; }
+// Bytes of the table of a layer of B sequences and NHl slabs, at an 8-byte
+// aligned base: OFF, P0 (both only when cached), NA, NP.
+__host__ __device__ constexpr int seq_table_bytes(int B, int NHl)
+{
+    return (NHl < kSlabCache ? NHl * 12 + 4 : 0) + (2 * B + 1) * 4;
+}
+// The most any layer of B sequences needs.
+__host__ __device__ constexpr int seq_table_bytes(int B) { return seq_table_bytes(B, kSlabCache - 1); }
 
 __device__ __forceinline__ SeqTable seq_table_at(unsigned char* base, const DecodeArgs& a)
 {
     SeqTable t;
-    const bool cached = a.B * a.Hkv < kSlabCache;
+    const int NHl = a.B * a.Hkv;
+    const bool cached = NHl < kSlabCache;
     t.OFF = cached ? reinterpret_cast<int64_t*>(base) : nullptr;
-    t.IO = cached ? reinterpret_cast<int32_t*>(base + kSlabCache * 8) : nullptr;
-    t.NA = reinterpret_cast<int32_t*>(base + kSlabCache * 12);
+    t.P0 = cached ? reinterpret_cast<int32_t*>(base + NHl * 8) : nullptr;
+    t.NA = reinterpret_cast<int32_t*>(base + (cached ? NHl * 12 + 4 : 0));
     t.NP = t.NA + a.B;
     return t;
 }
 
-// Fill IO and OFF (when cached) with the threads [t0, t0 + nt) of the CTA; the
-// caller's barrier publishes them.
+// Fill P0 (context rows only, so far) and OFF (when cached) with the threads
+// [t0, t0 + nt) of the CTA; the caller's barrier publishes them.
 __device__ __forceinline__ void load_slab_cache(const DecodeArgs& a, SeqTable t, int t0, int nt)
 {
-    if (!t.IO) return;
+    if (!t.P0) return;
     const int NHl = a.B * a.Hkv;
     const int64_t i0 = __ldg(a.ioff);
+#pragma unroll 1
     for (int h = (int)threadIdx.x - t0; h <= NHl; h += nt) {
-        t.IO[h] = (int)(__ldg(a.ioff + h) - i0);
+        t.P0[h] = (int)(__ldg(a.ioff + h) - i0);
         if (h < NHl) t.OFF[h] = __ldg(a.off + h);
     }
+}
+
+// Rows that come before slab h in the layer beyond the context rows: NP is ready.
+__device__ __forceinline__ int extra_before(const int32_t* NP, int Hkv, int h)
+{
+    const int b = h / Hkv, g = h - b * Hkv;
+    int p = Hkv * NP[b];
+    if (g) p += g * (NP[b + 1] - NP[b]);
+    return p;
+}
+
+// After the barrier that publishes NP and P0's context rows: P0 becomes the
+// slabs' first layer rows (all nt threads of the CTA; the caller's next barrier
+// publishes it).
+__device__ __forceinline__ void finish_slab_cache(const DecodeArgs& a, SeqTable t, int nt)
+{
+    if (!t.P0) return;
+#pragma unroll 1
+    for (int h = threadIdx.x; h <= a.B * a.Hkv; h += nt) t.P0[h] += extra_before(t.NP, a.Hkv, h);
 }
 
 __device__ void build_seq_table(const DecodeArgs& a, SeqTable t, bool report)
@@ -83,6 +116,7 @@ __device__ void build_seq_table(const DecodeArgs& a, SeqTable t, bool report)
     // Called by one full warp.
     const int lane = threadIdx.x & 31;
     int carry = 0;
+#pragma unroll 1
     for (int b0 = 0; b0 < a.B; b0 += 32) {
         const int b = b0 + lane;
         int na = 0, e = 0;
@@ -107,13 +141,24 @@ __device__ void build_seq_table(const DecodeArgs& a, SeqTable t, bool report)
 }
 
 // First layer row of slab h (h in [0, B*Hkv]) within this call.
+// (Out of line, where the registers allow a call: its code would otherwise be
+// repeated at every use.)
+#ifndef DKV_SLAB_CALL
+#define DKV_SLAB_CALL __noinline__
+#endif
+__device__ DKV_SLAB_CALL int slab_start_global(const int64_t* ioff, const int32_t* NP, int Hkv, int h)
+{
+    return (int)(ioff[h] - ioff[0]) + extra_before(NP, Hkv, h);
+}
+
 __device__ __forceinline__ int slab_start(const DecodeArgs& a, const SeqTable& t, int h)
 {
-    const int b = h / a.Hkv, g = h - b * a.Hkv;
-    int p = (t.IO ? t.IO[h] : (int)(a.ioff[h] - a.ioff[0])) + a.Hkv * t.NP[b];
-    if (g) p += g * (t.NP[b + 1] - t.NP[b]);
-    return p;
+    return t.P0 ? t.P0[h] : slab_start_global(a.ioff, t.NP, a.Hkv, h);
 }
+
+// CTAs that get rows when R > 0 rows are cut into at most P ranges: the first
+// live_parts of the grid, each with at least one row.
+__device__ __forceinline__ int live_parts(int R, int P) { return min(P, max(R, 1)); }
 
 __device__ __forceinline__ int part_start(int w, int R, int P)
 {
@@ -131,7 +176,9 @@ __device__ __forceinline__ int part_of(int x, int R, int P)
 {
     const int64_t num = (int64_t)(x + 1) * P - 1;
     int w = (int)((float)num * __fdividef(1.f, (float)R));
+#pragma unroll 1
     while ((int64_t)(w + 1) * R <= num) ++w;
+#pragma unroll 1
     while (w > 0 && (int64_t)w * R > num) --w;
     return min(w, P - 1);
 }
@@ -140,6 +187,7 @@ __device__ __forceinline__ int part_of(int x, int R, int P)
 __device__ int slab_containing(const DecodeArgs& a, const SeqTable& t, int NHl, int x)
 {
     int lo = 0, hi = NHl - 1;
+#pragma unroll 1
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (slab_start(a, t, mid) <= x)
@@ -172,6 +220,7 @@ struct Cursor {
 __device__ __forceinline__ void cursor_seek(Cursor& cu, const DecodeArgs& a, const SeqTable& t, int hend, int wA,
                                             int wB)
 {
+#pragma unroll 1
     while (cu.h < hend) {
         cu.p0 = slab_start(a, t, cu.h);
         const int p1 = slab_start(a, t, cu.h + 1);
@@ -180,7 +229,7 @@ __device__ __forceinline__ void cursor_seek(Cursor& cu, const DecodeArgs& a, con
         if (cu.s0 < cu.s1) {
             const int b = cu.h / a.Hkv;
             const int e = t.NP[b + 1] - t.NP[b];
-            cu.n_h = (t.IO ? t.IO[cu.h + 1] - t.IO[cu.h] : a.len[cu.h]) + e;
+            cu.n_h = p1 - cu.p0;
             cu.app = (a.append && e > t.NA[b]) ? 1 : 0;
             cu.base = t.OFF ? t.OFF[cu.h] : a.off[cu.h];
             cu.x = cu.s0;
@@ -201,18 +250,13 @@ __device__ __forceinline__ void cursor_next(Cursor& cu, const DecodeArgs& a, con
 }
 
 // Number of CTAs whose row range overlaps [p0, p1) (p0 < p1), and the first and
-// last of them.
+// last of them (R >= P: every CTA has rows).
 __device__ __forceinline__ int ctas_of_slab(int p0, int p1, int R, int P, int* c0_out, int* c1_out)
 {
     const int c0 = part_of(p0, R, P), c1 = part_of(p1 - 1, R, P);
-    int n = c1 - c0 + 1;
-    if (R < P) {  // some CTAs have no rows (never when every CTA gets at least one)
-        n = 0;
-        for (int cc = c0; cc <= c1; ++cc) n += part_start(cc, R, P) < part_start(cc + 1, R, P) ? 1 : 0;
-    }
     *c0_out = c0;
     *c1_out = c1;
-    return n;
+    return c1 - c0 + 1;
 }
 
 // Output row of column c of slab (b, g): query c / G, head g G + c % G of out [B][Q][H][128].
@@ -232,84 +276,214 @@ __device__ __forceinline__ void write_out(const DecodeArgs& a, int b, int g, int
     dst[lane] = make_float4(O.x * inv, O.y * inv, O.z * inv, O.w * inv);
 }
 
-// Fused combine of head j of slab h by one warp of the last CTA to finish the
-// slab: the CTA partials in slots c + h, c in [c0, c1], which come from other
-// SMs (L2 loads). Every lane loads the (m, l) and its 4 dims of o of KB partials
-// at once, then merges them in registers; batches chain online. Measured: a
-// load round at the end of a launch takes ~1.5 us and grows with the bytes in
-// flight, so one round of 20-24 partials costs more than two smaller ones; of
-// 8, 10, 12, 16, 20 and 24, KB = 12 was fastest.
-template <int G, int KB, int NCC>
-__device__ void merge_slab_head(const DecodeArgs& a, int h, int j, int c0, int c1, int R, int lane)
+// ------------------------------------------------------------ cross-CTA merge
+// A slab whose rows lie in several CTAs is merged by the last of them (by index):
+// every other CTA leaves its partial (m, l, o) of a column in the fused-merge
+// exchange, slot c + h, and the merging CTA polls the slots until every word has
+// arrived. A slot's words carry their own arrival: an empty word is 0, and a
+// partial's zeros are written as -0, so a word is data as soon as it differs from
+// 0, whatever order the stores arrive in. That takes one store and one load
+// through L2, where an arrival counter took a fence, an atomic, an acquire and
+// then the loads: at 32K (50 MB layers) 9.3 us of streaming was followed by up
+// to 5.1 us of merge, now 3.3. The merging CTA empties the slots again for the
+// next launch (ordered by the launches' dependency). It waits only for CTAs of
+// lower index, which start no later than it does.
+__device__ __forceinline__ float full_word(float x) { return __float_as_uint(x) == 0u ? -0.f : x; }
+
+__device__ __forceinline__ bool is_full(const float4& v)
 {
-    const int b = h / a.Hkv, g = h - b * a.Hkv;
-    const int P = a.nctas;
-    const bool all_live = R >= P;
-    float M = -INFINITY, L = 0.f;
-    float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k0 = c0; k0 <= c1; k0 += KB) {
-        float2 ml[KB];
+    return __float_as_uint(v.x) != 0u && __float_as_uint(v.y) != 0u && __float_as_uint(v.z) != 0u &&
+           __float_as_uint(v.w) != 0u;
+}
+
+__device__ __forceinline__ float4 ld_exchange4(const float* p)
+{
+    float4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
+
+__device__ __forceinline__ float2 ld_exchange2(const float* p)
+{
+    float2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_exchange4(float* p, float4 v)
+{
+    asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                 : "memory");
+}
+
+__device__ __forceinline__ void st_exchange2(float* p, float x, float y)
+{
+    asm volatile("st.relaxed.gpu.global.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(x), "f"(y) : "memory");
+}
+
+// Bound of a poll loop over the exchange, decided by the whole warp: true once the
+// polls or the time since the 64th poll run out.
+__device__ __forceinline__ bool polled_out(int spin, unsigned long long& t0)
+{
+    if ((spin & 63) != 0) return false;
+    const unsigned long long now = global_ns();
+    if (t0 == 0) t0 = now;
+    return __any_sync(kFull, spin >= kWaitSpins || now - t0 > kWaitNs);
+}
+
+// One warp writes a CTA's partial of one column: slot index sj = (c + h) NC + j.
+__device__ __forceinline__ void put_partial(const DecodeArgs& a, int64_t sj, float4 O, float M, float L, int lane)
+{
+    st_exchange4(a.exch_o + sj * kHeadDim + 4 * lane,
+                 make_float4(full_word(O.x), full_word(O.y), full_word(O.z), full_word(O.w)));
+    if (lane == 0) st_exchange2(a.exch_ml + sj * 2, full_word(M), full_word(L));
+}
+
+// One warp of the merging CTA adds to a state (M, L, O: 4 dims a lane) of column
+// j of slab h the partials of the CTAs first, first + step, ... below end (step 1
+// or 2), KB at a time, and empties their slots. A batch is one round trip to L2
+// (0.5 us) once its words are there: lane k reads the k-th partial's m and l,
+// every lane its dims of all of them. KB = 12: with 8 a slab of 19 CTAs takes a
+// second round (128K 1,026 -> 1,040 us per step, 4K 261 -> 280), 16 is no faster.
+// False when a partial did not arrive within the wait bound.
+template <int KB, int NCC>
+__device__ __forceinline__ bool merge_partials(const DecodeArgs& a, int h, int j, int NC_, int first, int step,
+                                               int end, float& M, float& L, float4& O, int lane)
+{
+    const int NC = NCC ? NCC : NC_;
+    const int stride = step * NC;
+    const int64_t base = ((int64_t)first + h) * NC + j;
+    float* po = a.exch_o + base * kHeadDim + 4 * lane;
+    float* pm = a.exch_ml + (base + (int64_t)lane * stride) * 2;
+    bool good = true;
+    float Lk = 0.f;  // this lane's share of the partials' sums
+#pragma unroll 1
+    for (int n = (end - first + step - 1) >> (step - 1); n > 0;
+         n -= KB, po += KB * stride * kHeadDim, pm += KB * stride * 2) {
         float4 v[KB];
+        float2 ml;
+        unsigned long long t0 = 0;
+#pragma unroll 1
+        for (int spin = 1;; ++spin) {
+            ml = make_float2(-INFINITY, -0.f);
+            if (lane < min(n, KB)) ml = ld_exchange2(pm);
+            // Slots past the last one read the first again: no branches.
 #pragma unroll
-        for (int u = 0; u < KB; ++u) {
-            const int cc = k0 + u;
-            const bool ok = cc <= c1 && (all_live || part_start(cc, R, P) < part_start(cc + 1, R, P));
-            const int64_t sj = ((int64_t)cc + h) * (NCC ? NCC : a.NC) + j;
-            ml[u] = ok ? __ldcg(reinterpret_cast<const float2*>(a.work_ml + sj * 2)) : make_float2(-INFINITY, 0.f);
-            v[u] = ok ? __ldcg(reinterpret_cast<const float4*>(a.work_o + sj * kHeadDim) + lane)
-                      : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int u = 0; u < KB; ++u) v[u] = ld_exchange4(po + (u < n ? u * stride * kHeadDim : 0));
+            bool full = __float_as_uint(ml.x) != 0u && __float_as_uint(ml.y) != 0u;
+#pragma unroll
+            for (int u = 0; u < KB; ++u) full &= is_full(v[u]);
+            if (__all_sync(kFull, full)) break;
+            if (polled_out(spin, t0)) {
+                good = false;
+                break;
+            }
         }
-        float Mb = M;
+        float Mb = fmaxf(M, ml.x);
 #pragma unroll
-        for (int u = 0; u < KB; ++u) Mb = fmaxf(Mb, ml[u].x);
+        for (int o = 16; o >= 1; o >>= 1) Mb = fmaxf(Mb, __shfl_xor_sync(kFull, Mb, o));
         const float fo = (M == -INFINITY) ? 0.f : ex2(M - Mb);
+        const float f = (ml.x == -INFINITY) ? 0.f : ex2(ml.x - Mb);
+        M = Mb;
         L *= fo;
+        Lk = fmaf(Lk, fo, f * ml.y);
         O.x *= fo;
         O.y *= fo;
         O.z *= fo;
         O.w *= fo;
 #pragma unroll
         for (int u = 0; u < KB; ++u) {
-            const float f = (ml[u].x == -INFINITY) ? 0.f : ex2(ml[u].x - Mb);
-            L = fmaf(f, ml[u].y, L);
-            O.x = fmaf(f, v[u].x, O.x);
-            O.y = fmaf(f, v[u].y, O.y);
-            O.z = fmaf(f, v[u].z, O.z);
-            O.w = fmaf(f, v[u].w, O.w);
+            const float fu = __shfl_sync(kFull, f, u);
+            if (u < n) {
+                O.x = fmaf(fu, v[u].x, O.x);
+                O.y = fmaf(fu, v[u].y, O.y);
+                O.z = fmaf(fu, v[u].z, O.z);
+                O.w = fmaf(fu, v[u].w, O.w);
+                st_exchange4(po + u * stride * kHeadDim, make_float4(0.f, 0.f, 0.f, 0.f));
+            }
         }
-        M = Mb;
+        if (lane < min(n, KB)) st_exchange2(pm, 0.f, 0.f);
     }
-    write_out<G>(a, b, g, j, O, L, lane);
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) Lk += __shfl_xor_sync(kFull, Lk, o);
+    L += Lk;
+    if (!good && lane == 0) atomicOr(a.status, 0x4 /* DKV_DEV_MERGE_TIMEOUT */);
+    return good;
 }
 
-// End of one CTA's split-K pass, after its warps' ranges are done and a CTA
-// barrier. NCC: the number of columns per slab when fixed at compile time (the
-// decode step: G), 0 to take a.NC. meta: seg_first[NW], seg_last[NW] (first / last slab of warp w, -1 if
-// none), then the layer rows [p0, p1) of each entry (2 w: first, 2 w + 1: last)
-// as p0[2 NW], p1[2 NW], recorded while streaming so the end of the pass reads
-// no plan metadata from global memory;
-// the first slab's state is in the warp record (c, w) of warp_o / warp_ml, the
-// last slab's in warp w's own ring at ring + w * warp_ring_bytes (o[G][128] then
-// (m, l)[G]). The states of each slab are merged; a slab wholly inside this CTA
-// is written out (fused), otherwise the CTA writes its partial to slot c + h.
-// Fused, the CTA counts itself in for each (slab, head) before merging its
-// warps' states; the last CTA to arrive waits until the others have written
-// their partials and merges them all. A CTA writes its partial right after it
-// arrives, with no wait in between, so the last arriver's wait always ends.
-template <int G, int NW, bool FUSED, int NCC>
-__device__ void cta_tail(const DecodeArgs& a, const unsigned char* ring, int warp_ring_bytes,
-                         const int32_t* meta, int c, int R, int warp, int lane)
+// End of a CTA's pass after a copy that never landed: its outputs stay unwritten
+// (the status word says so), but the slabs it shares with other CTAs still get
+// their exchange words, as an empty partial, or are collected, so that no other
+// CTA waits for this one and the next launch finds the exchange empty.
+template <int NW>
+__device__ __noinline__ void dead_tail(const DecodeArgs& a, const SeqTable& tab, int NC, int c, int A, int Bc, int R,
+                                       int P, int warp, int lane)
 {
-    const int32_t* seg_first = meta;
-    const int32_t* seg_last = meta + NW;
-    const int32_t* seg_p0 = meta + 2 * NW;
-    const int32_t* seg_p1 = meta + 4 * NW;
+    const int NHl = a.B * a.Hkv;
+    const int hf = slab_containing(a, tab, NHl, A), hl = slab_containing(a, tab, NHl, Bc - 1);
+#pragma unroll 1
+    for (int e = 1; e >= 0; --e) {  // the last slab first: its partial waits for nobody
+        const int h = e ? hl : hf;
+        if (e && hl == hf) continue;
+        int c0, c1;
+        if (ctas_of_slab(slab_start(a, tab, h), slab_start(a, tab, h + 1), R, P, &c0, &c1) <= 1) continue;
+#pragma unroll 1
+        for (int j = warp; j < NC; j += NW) {
+            float M = -INFINITY, L = 0.f;
+            float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c1 == c)
+                merge_partials<4, 0>(a, h, j, NC, c0, 1, c1, M, L, O, lane);
+            else
+                put_partial(a, ((int64_t)c + h) * NC + j, O, M, L, lane);
+        }
+    }
+}
+
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+// What a CTA records for its end (int32 words in shared memory): seg_first[NW],
+// seg_last[NW] (first / last slab of warp w, -1 if none), the layer rows [p0, p1)
+// of each entry (2 w: first, 2 w + 1: last) as p0[2 NW], p1[2 NW], whether a warp
+// gave up a copy wait, and the first CTA of the CTA's first slab.
+template <int NW>
+struct TailMeta {
+    static constexpr int kFirst = 0, kLast = NW, kP0 = 2 * NW, kP1 = 4 * NW, kDead = 6 * NW, kC0 = 6 * NW + 1;
+    static constexpr int kWords = 6 * NW + 4;
+};
+
+// End of one CTA's split-K pass over the layer rows [A, Bc), after its warps'
+// ranges are done and a CTA barrier. NCC: the number of columns per slab when
+// fixed at compile time (the decode step: G), 0 to take a.NC. The first slab's
+// state of warp w is in the warp record (c, w) of warp_o / warp_ml, the last
+// slab's in its own ring at ring + w * ring_bytes (o[NC][128] then (m, l)[NC]);
+// the ring has 528 free bytes at dep_off. The states of each slab are merged; a
+// slab wholly inside this CTA is written out (fused). Otherwise the CTA leaves its partial in the exchange,
+// or, as the slab's last CTA, merges everyone's; not fused, the CTA writes its
+// partial to slot c + h of the workspace.
+//
+// A task is (slab, column), one warp each: it merges the CTA's own states. While
+// there are at least twice (three times) as many warps as tasks, a task has one
+// (two) more warps, which meanwhile collect the other CTAs' partials. With fewer
+// warps the tasks run from the CTA's last slab to its first, the only one it can
+// be the last CTA of: what others wait for is written before this CTA waits.
+template <int G, int NW, bool FUSED, int NCC>
+__device__ __forceinline__ void cta_tail(const DecodeArgs& a, unsigned char* ring, int ring_bytes, int dep_off,
+                                         const int32_t* meta, int c, int A, int Bc, int warp, int lane)
+{
+    using TM = TailMeta<NW>;
     // Entry e (lane e) is the first (even e) or last (odd e) slab of warp e/2, -1 if
-    // none; entries list their slabs in non-decreasing order. Task t = (slab #t/G,
-    // head t%G) for the distinct slabs; warp w takes tasks w, w+NW, ...
+    // none; entries list their slabs in non-decreasing order.
     static_assert(2 * NW <= 32, "one entry per lane");
-    const int h_e = (lane < 2 * NW) ? ((lane & 1) ? seg_last[lane >> 1] : seg_first[lane >> 1]) : -1;
-    const int p0_e = h_e >= 0 ? seg_p0[lane] : 0, p1_e = h_e >= 0 ? seg_p1[lane] : 0;
+    int h_e = -1, p0_e = 0, p1_e = 0;
+    if (lane < 2 * NW) {
+        h_e = meta[((lane & 1) ? TM::kLast : TM::kFirst) + (lane >> 1)];
+        p0_e = meta[TM::kP0 + lane];
+        p1_e = meta[TM::kP1 + lane];
+    }
     // Slab of the nearest valid entry before this one (-1 if none): one ballot
     // and one shuffle.
     const unsigned valid = __ballot_sync(kFull, h_e >= 0);
@@ -317,95 +491,121 @@ __device__ void cta_tail(const DecodeArgs& a, const unsigned char* ring, int war
     const int hprev = __shfl_sync(kFull, h_e, below ? 31 - __clz(below) : 0);
     const int prev = below ? hprev : -1;
     const unsigned fresh = __ballot_sync(kFull, h_e >= 0 && h_e != prev);
-    const int nslab = __popc(fresh);
+    const int nslab = uniform(__popc(fresh));
     const int NC = NCC ? NCC : a.NC;  // columns (query x head) per slab; NCC: known at compile time
-    // Task t = (slab #si, column j), t = si NC + j; warp w takes t = w, w + NW, ...
-    // (si, j) advance by additions: no division on this latency-bound path.
-    int si = 0, j = warp - NW;
-    for (int t = warp; t < nslab * NC; t += NW) {
-        j += NW;
-        while (j >= NC) {
-            j -= NC;
-            ++si;
+    const int T = nslab * NC;
+    const int team = !FUSED || 2 * T > NW ? 1 : 3 * T > NW ? 2 : 3;  // warps a task
+    int member = 0, first_task = warp;
+    if (team > 1) {
+        if (warp >= team * T) return;
+        member = warp >= 2 * T ? 2 : warp >= T ? 1 : 0;
+        first_task = warp - member * T;
+    }
+    // Tasks from the last: task t is (slab #si, column j); (si, j) go back by
+    // subtractions: no division on this latency-bound path.
+    int si = nslab - 1, j = NC - 1 - first_task;
+#pragma unroll 1
+    for (int t = T - 1 - first_task; t >= 0; t -= NW, j -= NW) {
+#pragma unroll 1
+        while (j < 0) {
+            j += NC;
+            --si;
         }
         unsigned m = fresh;
+#pragma unroll 1
         for (int k = 0; k < si; ++k) m &= m - 1;
-        const int e0 = __ffs(m) - 1;
-        const int h = __shfl_sync(kFull, h_e, e0);
-        const int hp0 = __shfl_sync(kFull, p0_e, e0), hp1 = __shfl_sync(kFull, p1_e, e0);
-        const unsigned same = __ballot_sync(kFull, h_e == h);
-        int c0h = 0, c1h = 0;
-        const int nct = FUSED ? ctas_of_slab(hp0, hp1, R, a.nctas, &c0h, &c1h) : 0;
-        // Count this CTA in for (slab, head) now, so that the atomic's round trip
-        // overlaps the merge below. Counter pair: arrivals, then partials written.
-        int32_t* ctr = FUSED ? a.slab_count + ((int64_t)h * NC + j) * 2 : nullptr;
-        int old = 0;
-        if (FUSED && nct > 1 && lane == 0)
-            asm volatile("atom.relaxed.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(ctr) : "memory");
-        float M = -INFINITY;
-#pragma unroll
-        for (int f = 0; f < 2 * NW; ++f) {
-            if (!((same >> f) & 1u)) continue;
-            const int w = f >> 1;
-            const float* ml = (f & 1) ? reinterpret_cast<const float*>(ring + w * warp_ring_bytes) + NC * kHeadDim
-                                      : a.warp_ml + ((int64_t)c * NW + w) * NC * 2;
-            M = fmaxf(M, ml[2 * j]);
-        }
+        const int e0 = uniform(__ffs(m) - 1);
+        const int h = uniform(__shfl_sync(kFull, h_e, e0));
+        const bool before = uniform(__shfl_sync(kFull, p0_e, e0) < A) != 0, after = uniform(__shfl_sync(kFull, p1_e, e0) > Bc) != 0;
+        const bool merger = FUSED && before && !after;  // this CTA is the slab's last of several
+        if (member > 0 && !merger) return;
+        float M = -INFINITY, L = 0.f;
         float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
-        float L = 0.f;
+        if (member == 0) {
+            // Lane e holds (m, l) of entry e when it is of this slab: odd entries in the
+            // warps' rings, even ones (at most one in a CTA whose slabs are longer than a
+            // warp's range) in the warp records.
+            const unsigned same = __ballot_sync(kFull, h_e == h);
+            const float* rf = reinterpret_cast<const float*>(ring);
+            const int ring_floats = ring_bytes / 4;
+            float2 ml = make_float2(-INFINITY, 0.f);
+            if (h_e == h)
+                ml = *reinterpret_cast<const float2*>(
+                    (lane & 1) ? rf + (lane >> 1) * ring_floats + NC * kHeadDim + 2 * j
+                               : a.warp_ml + (((int64_t)c * NW + (lane >> 1)) * NC + j) * 2);
+            M = ml.x;
 #pragma unroll
-        for (int f = 0; f < 2 * NW; ++f) {
-            if (!((same >> f) & 1u)) continue;
-            const int w = f >> 1;
-            const float* ob = (f & 1) ? reinterpret_cast<const float*>(ring + w * warp_ring_bytes)
-                                      : a.warp_o + ((int64_t)c * NW + w) * NC * kHeadDim;
-            const float* ml = (f & 1) ? ob + NC * kHeadDim : a.warp_ml + ((int64_t)c * NW + w) * NC * 2;
-            const float2 mlj = *reinterpret_cast<const float2*>(ml + 2 * j);
-            const float fct = (mlj.x == -INFINITY) ? 0.f : ex2(mlj.x - M);
-            L = fmaf(mlj.y, fct, L);
-            const float4 v = reinterpret_cast<const float4*>(ob + j * kHeadDim)[lane];
-            O.x = fmaf(v.x, fct, O.x);
-            O.y = fmaf(v.y, fct, O.y);
-            O.z = fmaf(v.z, fct, O.z);
-            O.w = fmaf(v.w, fct, O.w);
-        }
-        if (FUSED && nct == 1) {
-            write_out<G>(a, h / a.Hkv, h % a.Hkv, j, O, L, lane);  // the slab lies wholly in this CTA
-            continue;
-        }
-        const int64_t slot = (int64_t)c + h;
-        reinterpret_cast<float4*>(a.work_o + (slot * NC + j) * kHeadDim)[lane] = O;
-        if (lane == 0) *reinterpret_cast<float2*>(a.work_ml + (slot * NC + j) * 2) = make_float2(M, L);
-        if (!FUSED) continue;
-        __syncwarp();
-        if (__shfl_sync(kFull, old, 0) != nct - 1) {
-            // Not the last: release the partial just written to the last arriver.
-            if (lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(ctr + 1) : "memory");
-            continue;
-        }
-        // The last arriver: acquire the other CTAs' partials once all are written
-        // (a bounded wait: every CTA that arrived is resident and writes next),
-        // make the counters ready for the next call, and merge.
-        int ok = 1;
-        if (lane == 0) {
-            ok = 0;
-            const unsigned long long t0 = global_ns();
-            for (int i = 1; i < kWaitSpins; ++i) {
-                int n;
-                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(n) : "l"(ctr + 1) : "memory");
-                if (n == nct - 1 + a.merge_extra) {
-                    ok = 1;
-                    break;
-                }
-                if ((i & 63) == 0 && global_ns() - t0 > kWaitNs) break;
+            for (int o = 16; o >= 1; o >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, o));
+            const float f = (ml.x == -INFINITY) ? 0.f : ex2(ml.x - M);
+            rf += j * kHeadDim + 4 * lane;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                const float fw = __shfl_sync(kFull, f, 2 * w + 1);  // 0 when the entry is not of this slab
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if ((same >> (2 * w + 1)) & 1u) v = *reinterpret_cast<const float4*>(rf + w * ring_floats);
+                O.x = fmaf(v.x, fw, O.x);
+                O.y = fmaf(v.y, fw, O.y);
+                O.z = fmaf(v.z, fw, O.z);
+                O.w = fmaf(v.w, fw, O.w);
             }
-            if (!ok) atomicOr(a.status, 0x4 /* DKV_DEV_MERGE_TIMEOUT */);
-            ctr[0] = 0;
-            ctr[1] = 0;
+#pragma unroll 1
+            for (unsigned e = uniform(same & 0x55555555u); e; e &= e - 1) {
+                const int w2 = __ffs(e) - 1;
+                const float fw = __shfl_sync(kFull, f, w2);
+                const float4 v = reinterpret_cast<const float4*>(
+                    a.warp_o + (((int64_t)c * NW + (w2 >> 1)) * NC + j) * kHeadDim)[lane];
+                O.x = fmaf(v.x, fw, O.x);
+                O.y = fmaf(v.y, fw, O.y);
+                O.z = fmaf(v.z, fw, O.z);
+                O.w = fmaf(v.w, fw, O.w);
+            }
+            L = f * ml.y;
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) L += __shfl_xor_sync(kFull, L, o);
         }
-        ok = __shfl_sync(kFull, ok, 0);
-        __syncwarp();
-        if (ok) merge_slab_head<G, 12, NCC>(a, h, j, c0h, c1h, R, lane);
+        const int64_t sj = ((int64_t)c + h) * NC + j;
+        if (!FUSED) {
+            reinterpret_cast<float4*>(a.work_o + sj * kHeadDim)[lane] = O;
+            if (lane == 0) *reinterpret_cast<float2*>(a.work_ml + sj * 2) = make_float2(M, L);
+            continue;
+        }
+        if (after) {
+            put_partial(a, sj, O, M, L, lane);
+            continue;
+        }
+        bool good = true;
+        if (merger) {
+            float* dep = reinterpret_cast<float*>(ring + warp * ring_bytes + dep_off);
+            if (team == 1 || member > 0)
+                good = merge_partials<12, NCC>(a, h, j, NC, meta[TM::kC0] + max(member - 1, 0), team == 3 ? 2 : 1,
+                                                   c + a.merge_extra, M, L, O, lane);
+            if (member > 0) {
+                reinterpret_cast<float4*>(dep)[lane] = O;
+                if (lane == 0) *reinterpret_cast<float4*>(dep + kHeadDim) = make_float4(M, L, good ? 1.f : 0.f, 0.f);
+                bar_arrive(1 + t, 32 * team);
+                return;
+            }
+            if (team > 1) {
+                bar_sync(1 + t, 32 * team);
+#pragma unroll
+                for (int k = 1; k <= 2; ++k) {
+                    if (k >= team) break;
+                    const float* d = dep + k * T * (ring_bytes / 4);
+                    const float4 v = reinterpret_cast<const float4*>(d)[lane];
+                    const float4 ml = *reinterpret_cast<const float4*>(d + kHeadDim);
+                    good &= ml.z != 0.f;
+                    const float Mb = fmaxf(M, ml.x);
+                    const float f0 = (M == -INFINITY) ? 0.f : ex2(M - Mb), f1 = (ml.x == -INFINITY) ? 0.f : ex2(ml.x - Mb);
+                    M = Mb;
+                    L = fmaf(ml.y, f1, L * f0);
+                    O.x = fmaf(v.x, f1, O.x * f0);
+                    O.y = fmaf(v.y, f1, O.y * f0);
+                    O.z = fmaf(v.z, f1, O.z * f0);
+                    O.w = fmaf(v.w, f1, O.w * f0);
+                }
+            }
+        }
+        if (good) write_out<G>(a, h / a.Hkv, h % a.Hkv, j, O, L, lane);
     }
 }
 

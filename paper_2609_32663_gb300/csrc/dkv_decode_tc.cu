@@ -58,6 +58,7 @@
 // without work, so that they still meet at every named barrier), the copies and
 // products in flight are drained with the same bound, and TMEM is freed before
 // the CTA exits.
+#define DKV_SLAB_CALL __forceinline__
 #include "dkv_decode_common.cuh"
 
 #include <cuda.h>
@@ -452,6 +453,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         fence_proxy_async_smem();
     }
     __syncthreads();
+    finish_slab_cache(a, tab, kTcThreads);
+    __syncthreads();
     pdl_launch_dependents();
 
     const int R = slab_start(a, tab, NHl);
@@ -466,9 +469,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     TcPart part;
     part.R = R;
-    part.P = a.nctas;
+    part.P = live_parts(R, a.nctas);
     part.NHl = NHl;
-    part.scale = (float)a.nctas / (float)max(R, 1);
+    part.scale = (float)part.P / (float)max(R, 1);
     part.aligned = NHl * 4 <= a.nctas && R >= 4 * a.nctas;
     // Only while no CTA would get more than 1.15 shares of rows (R / P), and every
     // slab with rows gets a CTA of its own.
@@ -477,8 +480,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const int n = part.cb(a, tab, h + 1) - part.cb(a, tab, h);
         if (rows > 0 && (n < 1 || (float)rows * part.scale > 1.15f * (float)n)) part.aligned = false;
     }
+    if (c >= part.P || R < 1) return;  // uniform: this CTA has no rows (no TMEM taken yet)
     const int A = part.start(a, tab, c), Bc = part.start(a, tab, c + 1);
-    if (A >= Bc) return;  // uniform: this CTA has no rows (no TMEM taken yet)
     const int hfirst = slab_containing(a, tab, NHl, A);
     const int hend = slab_containing(a, tab, NHl, Bc - 1) + 1;
     const int NC = a.NC;
@@ -947,7 +950,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
         // ---- the CTA's share of the merges of its slabs that span several CTAs
         // (its first and its last segment; the slabs in between were whole).
-        const int P = a.nctas;
         for (int e = 0; e < 2; ++e) {
             const int h = e == 0 ? hfirst : hend - 1;
             if (e == 1 && h == hfirst) break;
@@ -978,15 +980,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             named_sync(kBarSoft, kTcSoft);
             if (flags[kFlagSegOk]) {
-                // Rank of this CTA among the slab's CTAs (every CTA of the range is live
-                // when the layer has at least one row per CTA).
-                const bool all_live = R >= P;
-                int k = 0;
-                if (all_live) {
-                    k = c - c0;
-                } else {
-                    for (int cc = c0; cc < c; ++cc) k += part.start(a, tab, cc) < part.start(a, tab, cc + 1) ? 1 : 0;
-                }
+                const int k = c - c0;  // rank of this CTA among the slab's CTAs
                 const int j0 = (int)((int64_t)k * NC / nct), j1 = (int)((int64_t)(k + 1) * NC / nct);
                 const int hb = h / a.Hkv, hg = h - hb * a.Hkv;
                 // Columns j0 .. j1-1: warp (gi, quarter) takes j0 + 4 gi + quarter, then
@@ -1000,7 +994,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
                     for (int k0 = 0; k0 < ncta; k0 += 32) {
                         const int cc = c0 + k0 + lane;
-                        const bool okp = cc <= c1 && (all_live || part.start(a, tab, cc) < part.start(a, tab, cc + 1));
+                        const bool okp = cc <= c1;
                         const float2 ml = okp ? __ldcg(reinterpret_cast<const float2*>(a.work_ml + (((int64_t)cc + h) * NC + j) * 2))
                                               : make_float2(-INFINITY, 0.f);
                         float rm = ml.x;

@@ -89,6 +89,8 @@ struct DecodeArgs {
     float* work_ml;         // [slots][G][2]
     float* warp_o;          // [nparts][G][128]: a warp's state for a slab it left mid-range
     float* warp_ml;         // [nparts][G][2]
+    float* exch_o;          // fused-merge exchange: [slots][NC][128] and [slots][NC][2], every word 0 between launches
+    float* exch_ml;
     float* out;             // [B][H][128]
     int32_t* slab_count;    // [B*Hkv][cols][2] arrivals, partials written (zero between calls)
     int32_t* status;
@@ -149,8 +151,8 @@ inline WorkspaceLayout decode_workspace(int nctas, int nwarps, int cols, int hea
 cudaError_t decode_config(int G, int B, DecodeConfig* cfg);
 // Split-K partials of one layer into the workspace, then the per-(b, q-head) merge.
 cudaError_t launch_decode_partial(const DecodeArgs& a, const DecodeConfig& cfg, cudaStream_t st);
-// The partial pass with the combine fused in: the last CTA to finish a slab merges
-// the slab's partials and writes out (uses a.slab_count).
+// The partial pass with the combine fused in: a slab's last CTA merges the slab's
+// partials and writes out (uses the exchange).
 cudaError_t launch_decode_fused(const DecodeArgs& a, const DecodeConfig& cfg, cudaStream_t st);
 cudaError_t launch_decode_combine(const DecodeArgs& a, cudaStream_t st);
 
@@ -164,11 +166,11 @@ struct CacheMaps {
 constexpr int64_t kMaxMmaRows = ((int64_t)1 << 31) - 16;
 // Boxes of box_rows rows x 64 dims (16 for the mma.sync kernels, 64 for the tcgen05 one).
 cudaError_t make_cache_maps(const void* Kc, const void* Vc, int64_t rows, CacheMaps* maps, bool short_boxes = false,
-                            int box_rows = 16);
+                            int box_rows = 16, bool halves = true);
 // Launch configuration of the tensor-core kernels of one kind: 0 = the decode
 // step (G columns), 1 = multi-query with one tile of 8 columns, 2 = multi-query
 // with two tiles (up to 16 columns).
-cudaError_t decode_config_mma(int G, int B, int kind, DecodeConfig* cfg);
+cudaError_t decode_config_mma(int G, int B, int Hkv, int kind, DecodeConfig* cfg);
 cudaError_t launch_decode_mma_partial(const DecodeArgs& a, const CacheMaps& maps, const DecodeConfig& cfg,
                                       cudaStream_t st);
 cudaError_t launch_decode_mma_fused(const DecodeArgs& a, const CacheMaps& maps, const DecodeConfig& cfg,

@@ -57,15 +57,19 @@ __device__ __forceinline__ unsigned long long global_ns()
 // Bounded wait: false when the phase did not complete within kWaitSpins polls
 // or kWaitNs nanoseconds, whichever comes first (a poll's suspension is
 // system-defined, so the count alone does not bound the time).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
+__device__ __noinline__ bool mbar_wait_more(uint32_t bar, uint32_t parity)
 {
-    if (mbar_try_wait(bar, parity)) return true;
     const unsigned long long t0 = global_ns();
     for (int i = 1; i < kWaitSpins; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((i & 63) == 0 && global_ns() - t0 > kWaitNs) return false;
     }
     return false;
+}
+
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
+{
+    return mbar_try_wait(bar, parity) || mbar_wait_more(bar, parity);
 }
 
 __device__ __forceinline__ uint64_t evict_first_policy()

@@ -1,0 +1,82 @@
+"""The cross-CTA merge of the fused decode kernels: its edges and its values.
+
+A slab over several CTAs is merged by its last CTA from words that are 0 while
+empty, with one, two or three warps a (slab, column). Sizes here put it at its
+edges: fewer rows than CTAs, one row a CTA, slabs that end on a CTA boundary, one
+to many slabs a CTA; values that are exactly 0 (which must not read as "empty").
+Outputs against the fp64 oracle within the suite's tolerance; the constant-value
+cases against their closed form within 1e-5 (64 x the fp32 rounding of one sum).
+"""
+import pytest
+import torch
+
+import paper_2609_32663_gb300.dkv as dkv
+from paper_2609_32663_gb300 import inputs as I
+from parity import Case
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built(cuda):
+    from paper_2609_32663_gb300 import build
+    build.build_library()
+    torch.cuda.set_device(cuda)
+
+
+def wl(**kw):
+    base = dict(L=1, H=4, Hkv=1, T=3000, B=1, D=2, W=2000, pattern="ones", rate=1.0, seed=7)
+    base.update(kw)
+    return I.Workload("merge", **base)
+
+
+@pytest.mark.parametrize("G", [1, 4, 8])
+@pytest.mark.parametrize("T", [3, 75, 76, 151, 152, 153, 152 * 16, 152 * 16 + 1, 5000])
+def test_rows_around_the_cta_count(G, T):
+    c = Case(wl(H=G, T=T), reserve=2)
+    c.decode_steps(2, append=True)
+    c.close()
+
+
+@pytest.mark.parametrize("G,Hkv,B,T", [(4, 8, 1, 4096), (4, 2, 1, 4104), (7, 4, 4, 2000), (8, 1, 3, 1700),
+                                       (2, 19, 1, 1216), (1, 16, 16, 1300), (3, 5, 40, 1170)])
+def test_slabs_per_cta(G, Hkv, B, T):
+    """From one slab over many CTAs to many slabs a CTA (teams of three, two and one warps a task)."""
+    c = Case(wl(H=G * Hkv, Hkv=Hkv, B=B, T=T, seed=T), reserve=1)
+    c.decode_steps(1, append=True)
+    c.close()
+
+
+@pytest.mark.parametrize("G", [4, 7])
+@pytest.mark.parametrize("v", [0.0, 1.0])
+def test_zero_scores_and_constant_values(G, v):
+    """q = 0: every score and running max is exactly 0 and the output is V's mean."""
+    c = Case(wl(H=2 * G, Hkv=2, T=9000, W=4000))
+    q = torch.zeros((1, 2 * G, 128), dtype=torch.bfloat16, device=c.dev)
+    c.Vc.fill_(v)
+    out = torch.full((1, 2 * G, 128), float("nan"), device=c.dev)
+    for _ in range(3):
+        dkv.dkv_decode_attn(c.plan, 0, q, None, None, None, c.Kc, c.Vc, out)
+        assert (out - v).abs().max().item() <= 1e-5
+    assert dkv.dkv_plan_status(c.plan) == 0
+    c.close()
+
+
+def test_back_to_back_calls_are_identical():
+    """The exchange is empty again after every launch: calls in a row, over two
+    layers, with one and several queries, repeat their outputs bit for bit."""
+    c = Case(wl(L=2, H=8, Hkv=2, T=9000, W=4000, B=2))
+    q = I.decode_inputs(c.wl, 1)[0][0].to(c.dev)
+    qm = torch.stack([q, -q], dim=2)  # [L][B][2][H][128]
+    first = None
+    for _ in range(20):
+        outs = [torch.empty((2, 8, 128), device=c.dev) for _ in range(2)]
+        multi = [torch.empty((2, 2, 8, 128), device=c.dev) for _ in range(2)]
+        for l in range(2):
+            dkv.dkv_decode_attn(c.plan, l, q[l], None, None, None, c.Kc, c.Vc, outs[l])
+            dkv.dkv_decode_multi(c.plan, l, qm[l].contiguous(), 2, None, c.Kc, c.Vc, multi[l])
+        got = torch.cat([t.reshape(-1) for t in outs + multi])
+        first = got if first is None else first
+        assert torch.equal(got, first)
+    assert dkv.dkv_plan_status(c.plan) == 0
+    c.close()
