@@ -49,7 +49,7 @@ __device__ __forceinline__ void pdl_wait()
 // previous kernel has drained (the last ones to get an SM) would otherwise pay
 // a chain of dependent L2 round trips, under full HBM load, before its first
 // copy. P0 and OFF are null for larger layers (computed from global memory then).
-constexpr int kSlabCache = 1024;
+constexpr int kSlabCache = 1008;
 struct SeqTable {
     int32_t* NA;   // [B]
     int32_t* NP;   // [B+1]
@@ -141,12 +141,8 @@ __device__ void build_seq_table(const DecodeArgs& a, SeqTable t, bool report)
 }
 
 // First layer row of slab h (h in [0, B*Hkv]) within this call.
-// (Out of line, where the registers allow a call: its code would otherwise be
-// repeated at every use.)
-#ifndef DKV_SLAB_CALL
-#define DKV_SLAB_CALL __noinline__
-#endif
-__device__ DKV_SLAB_CALL int slab_start_global(const int64_t* ioff, const int32_t* NP, int Hkv, int h)
+// (Out of line: its code would otherwise be repeated at every use.)
+__device__ __noinline__ int slab_start_global(const int64_t* ioff, const int32_t* NP, int Hkv, int h)
 {
     return (int)(ioff[h] - ioff[0]) + extra_before(NP, Hkv, h);
 }
@@ -247,6 +243,57 @@ __device__ __forceinline__ void cursor_next(Cursor& cu, const DecodeArgs& a, con
     if (cu.x < cu.s1) return;
     ++cu.h;
     cursor_seek(cu, a, t, hend, wA, wB);
+}
+
+// ------------------------------------------------------------ segments
+// A warp's rows of one slab.
+struct Segment {
+    int h;      // slab
+    int left;   // rows (of the segment) from `row` on
+    int row;    // cache row of the first of them
+    int p0, p1; // the slab's layer rows
+    int app;    // the segment's last row is this step's new token
+};
+
+// The first segment of a slab in [h, hend), which has one, of a warp with the
+// layer rows [wA, wB), into the warp's slot in shared memory. (Returned that way,
+// not through a local variable: a stack frame of the decode kernels is more than
+// the L1 that their shared memory leaves, and a reload from L2 under full load
+// costs up to 1 us.)
+__device__ __noinline__ void find_segment(const DecodeArgs& a, unsigned char* table, int h, int hend, int wA, int wB,
+                                          int32_t* slot)
+{
+    const SeqTable t = seq_table_at(table, a);
+    int p0 = slab_start(a, t, h), p1 = p0;
+#pragma unroll 1
+    for (; h < hend; ++h, p0 = p1) {
+        p1 = slab_start(a, t, h + 1);
+        if (max(wA, p0) < min(wB, p1)) break;
+    }
+    const int s0 = max(wA, p0), s1 = min(wB, p1), b = h / a.Hkv;
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) {
+        slot[0] = h;
+        slot[1] = s1 - s0;
+        slot[2] = (int)((t.OFF ? t.OFF[h] : a.off[h]) + (s0 - p0));
+        slot[3] = p0;
+        slot[4] = p1;
+        slot[5] = (a.append && s1 == p1 && t.NP[b + 1] - t.NP[b] > t.NA[b]) ? 1 : 0;
+    }
+    __syncwarp();
+}
+
+__device__ __forceinline__ Segment read_segment(const int32_t* slot)
+{
+    return {uniform(slot[0]), uniform(slot[1]), uniform(slot[2]), uniform(slot[3]), uniform(slot[4]), uniform(slot[5])};
+}
+
+// Slabs of the warp's first and last row.
+__device__ __noinline__ int2 slab_range(const DecodeArgs& a, unsigned char* table, int wA, int wB)
+{
+    const SeqTable t = seq_table_at(table, a);
+    const int NHl = a.B * a.Hkv;
+    return make_int2(slab_containing(a, t, NHl, wA), slab_containing(a, t, NHl, wB - 1));
 }
 
 // Number of CTAs whose row range overlaps [p0, p1) (p0 < p1), and the first and

@@ -392,55 +392,6 @@ __device__ __noinline__ void zero_rows(unsigned char* st, int cnt, int lane)
     __syncwarp();
 }
 
-// A warp's rows of one slab.
-struct Segment {
-    int h;      // slab
-    int left;   // rows (of the segment) from `row` on
-    int row;    // cache row of the first of them
-    int p0, p1; // the slab's layer rows
-    int app;    // the segment's last row is this step's new token
-};
-
-// The warp's first segment of a slab in [h, hend), which has one, into the warp's
-// slot in shared memory. (Returned that way, not through a local variable: a
-// stack frame of this kernel is more than the L1 that its shared memory leaves,
-// and a reload from L2 under full load costs up to 1 us.)
-__device__ __noinline__ void find_segment(const DecodeArgs& a, unsigned char* table, int h, int hend, int wA, int wB,
-                                          int32_t* slot)
-{
-    const SeqTable t = seq_table_at(table, a);
-    int p0 = slab_start(a, t, h), p1 = p0;
-#pragma unroll 1
-    for (; h < hend; ++h, p0 = p1) {
-        p1 = slab_start(a, t, h + 1);
-        if (max(wA, p0) < min(wB, p1)) break;
-    }
-    const int s0 = max(wA, p0), s1 = min(wB, p1), b = h / a.Hkv;
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) {
-        slot[0] = h;
-        slot[1] = s1 - s0;
-        slot[2] = (int)((t.OFF ? t.OFF[h] : a.off[h]) + (s0 - p0));
-        slot[3] = p0;
-        slot[4] = p1;
-        slot[5] = (a.append && s1 == p1 && t.NP[b + 1] - t.NP[b] > t.NA[b]) ? 1 : 0;
-    }
-    __syncwarp();
-}
-
-__device__ __forceinline__ Segment read_segment(const int32_t* slot)
-{
-    return {uniform(slot[0]), uniform(slot[1]), uniform(slot[2]), uniform(slot[3]), uniform(slot[4]), uniform(slot[5])};
-}
-
-// Slabs of the warp's first and last row.
-__device__ __noinline__ int2 slab_range(const DecodeArgs& a, unsigned char* table, int wA, int wB)
-{
-    const SeqTable t = seq_table_at(table, a);
-    const int NHl = a.B * a.Hkv;
-    return make_int2(slab_containing(a, t, NHl, wA), slab_containing(a, t, NHl, wB - 1));
-}
-
 // The CTA that holds the first row of the slab of layer row A.
 __device__ __noinline__ void first_cta(const DecodeArgs& a, unsigned char* table, int A, int R, int P, int32_t* out)
 {

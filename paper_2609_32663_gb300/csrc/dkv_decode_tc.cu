@@ -10,13 +10,13 @@
 // other decode kernels. A CTA walks its range in tiles of 64 rows, slab segment
 // by slab segment (a segment: the part of one slab inside the CTA's range).
 //
-//   warp 0 (one lane)   TMA: a tile's K rows and V rows, each as 16-row 2-D
+//   warp 0              (one lane issues) TMA: a tile's K rows and V rows, each as 16-row 2-D
 //                       boxes (64 dims, 128-byte swizzle; measured faster than
 //                       64- or 32-row boxes), into separate
 //                       rings (4 K stages, 5 V stages): a K stage is released as
 //                       soon as its score product is done, a V stage only after
 //                       its output product, so V is the deeper ring.
-//   warp 1 (one lane)   MMA: S^T = Q K^T  (M = 64 query-column rows of Q, zero
+//   warp 1              (one lane issues) MMA: S^T = Q K^T  (M = 64 query-column rows of Q, zero
 //                       past the last column, N = 64 cache rows, K = 128 dims;
 //                       8 MMAs) into one of four TMEM score buffers, running up
 //                       to four tiles ahead of O^T += V^T P  (M = 128 dims, N =
@@ -53,12 +53,19 @@
 // (CTA k of the slab's nct CTAs takes columns k NC / nct .. (k+1) NC / nct):
 // the merge is spread over the slab's CTAs instead of falling on the last one.
 //
+// What bounds it: a 64-row tile is 32 KB, 0.73 us at an SM's share of HBM, and its
+// products need 0.3 us of the tensor pipe's operand bandwidth, so the schedules of
+// the roles set the pace. They run on warp-uniform values (uniform()): with a
+// single-lane MMA loop every operand went through a vector register and a move
+// before each product, and the kernel's code was 136 KB of walkers and partition
+// arithmetic, repeated inline, now 93. Same box, 4 layers at 128K: 64 columns 236
+// -> 189 us, 32 columns 229 -> 173; Qwen shape 64K x 4, 28 columns 250 -> 180.
+//
 // Every wait is bounded (polls and 2 s). A wait that runs out sets a
 // DKV_DEV_* bit, the roles stop (the softmax groups keep walking the tiles,
 // without work, so that they still meet at every named barrier), the copies and
 // products in flight are drained with the same bound, and TMEM is freed before
 // the CTA exits.
-#define DKV_SLAB_CALL __forceinline__
 #include "dkv_decode_common.cuh"
 
 #include <cuda.h>
@@ -100,7 +107,10 @@ constexpr int kOffBars = kOffFlags + 24 * 4;               // uint64 barriers
 // k_full[K], k_empty[K], v_full[V], v_empty[V], s_full[4], p_full[2], o_done[2], q_full[2], fin
 constexpr int kNumBars = 2 * kKStages + 2 * kVStages + kSBufs + 7;
 constexpr int kOffTmem = kOffBars + kNumBars * 8;
-constexpr int kOffTable = (kOffTmem + 16 + 15) / 16 * 16;
+constexpr int kOffInfo = kOffTmem + 16;                   // int[kInfoWords]: the CTA's share (TcShare)
+constexpr int kInfoWords = 8;
+constexpr int kOffSlots = kOffInfo + kInfoWords * 4;      // int[6] a warp: its current segment
+constexpr int kOffTable = (kOffSlots + kTcThreads / 32 * 24 + 15) / 16 * 16;
 constexpr int kTcAlign = 1024;
 __host__ __device__ constexpr int tc_smem_bytes(int B) { return kTcAlign + kOffTable + seq_table_bytes(B); }
 static_assert(tc_smem_bytes(kMaxB) <= 227 * 1024, "fits the opt-in shared memory of one CTA");
@@ -264,6 +274,14 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return d;
 }
 
+// One lane of a converged warp, the same each time.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // Bounded wait by one thread; true when the phase completed.
 __device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t parity) { return mbar_wait(smem_u32(bar), parity); }
 // One poll that never suspends the thread (mbarrier.try_wait may suspend it for a
@@ -282,38 +300,58 @@ __device__ __forceinline__ bool test_phase(uint64_t* bar, uint32_t parity)
     return ok != 0;
 }
 
+// test_phase by a whole warp.
+__device__ __forceinline__ bool test_phase_warp(uint64_t* bar, uint32_t parity)
+{
+    return __all_sync(kFull, test_phase(bar, parity));
+}
+
 // ------------------------------------------------------------ tiles
 // The CTA's tiles, slab segment by slab segment; tiles are 64 rows from the
-// segment's start.
+// segment's start. All of it is warp-uniform (see uniform()).
 struct TileWalk {
-    Cursor cu;
+    Segment sg;       // `left` and `row` run on tile by tile
     int hend, A, B;
-    __device__ void begin(const DecodeArgs& a, const SeqTable& t, int hfirst, int hend_, int A_, int B_)
+    int rows;         // of the whole segment
+    int32_t* slot;    // the warp's segment slot in shared memory
+    __device__ __forceinline__ void begin(const DecodeArgs& a, unsigned char* table, int hfirst, int hend_, int A_, int B_,
+                                          int32_t* slot_)
     {
         hend = hend_;
         A = A_;
         B = B_;
-        cu.h = hfirst;
-        cursor_seek(cu, a, t, hend, A, B);
+        slot = slot_;
+        seek(a, table, hfirst);
     }
-    __device__ bool more() const { return cu.h < hend; }
-    __device__ int cnt() const { return min(kTcRows, cu.s1 - cu.x); }
-    __device__ bool first() const { return cu.x == cu.s0; }
-    __device__ bool last() const { return cu.x + kTcRows >= cu.s1; }
-    __device__ int cache_row() const { return (int)(cu.base + (cu.x - cu.p0)); }
-    __device__ void next(const DecodeArgs& a, const SeqTable& t) { cursor_next<kTcRows>(cu, a, t, hend, A, B); }
+    __device__ __forceinline__ void seek(const DecodeArgs& a, unsigned char* table, int h)
+    {
+        find_segment(a, table, h, hend, A, B, slot);
+        sg = read_segment(slot);
+        rows = sg.left;
+    }
+    __device__ __forceinline__ bool more() const { return sg.left > 0; }
+    __device__ __forceinline__ int cnt() const { return min(kTcRows, sg.left); }
+    __device__ __forceinline__ bool first() const { return sg.left == rows; }
+    __device__ __forceinline__ bool last() const { return sg.left <= kTcRows; }
+    __device__ __forceinline__ int cache_row() const { return sg.row; }
+    __device__ __forceinline__ void next(const DecodeArgs& a, unsigned char* table)
+    {
+        sg.left -= kTcRows;
+        sg.row += kTcRows;
+        if (sg.left <= 0 && sg.h + 1 < hend) seek(a, table, sg.h + 1);
+    }
 };
 
-// Slab of the segment `skip` segments after the one under `cu` (>= hend when
-// there is none).
-__device__ __forceinline__ int later_segment_slab(Cursor cu, const DecodeArgs& a, const SeqTable& t, int hend, int A,
-                                                  int B, int skip)
+// Slab of the segment `skip` (1 or 2) segments after slab h's in the layer rows
+// [A, B) (hend when there is none; slabs up to hend - 1 have rows there or none).
+__device__ __noinline__ int later_segment_slab(const DecodeArgs& a, unsigned char* table, int h, int hend, int A, int B,
+                                               int skip)
 {
-    for (int k = 0; k < skip && cu.h < hend; ++k) {
-        ++cu.h;
-        cursor_seek(cu, a, t, hend, A, B);
-    }
-    return cu.h;
+    const SeqTable t = seq_table_at(table, a);
+#pragma unroll 1
+    for (++h; h < hend; ++h)
+        if (max(A, slab_start(a, t, h)) < min(B, slab_start(a, t, h + 1)) && --skip == 0) break;
+    return min(h, hend);
 }
 
 // Q of slab h as the A operand: row c (column c: query c / G, head g G + c % G)
@@ -411,6 +449,71 @@ struct TcPart {
     }
 };
 
+// A CTA's share of the layer: its rows [A, Bc), first and last slab, and for both
+// the CTAs they lie in (their first, and their count).
+struct TcShare {
+    int A, Bc, hfirst, hlast, c0_first, n_first, c0_last, n_last;
+};
+static_assert(sizeof(TcShare) == kInfoWords * 4, "the info words");
+
+// One warp computes it for the CTA (A = Bc: no rows). Out of line and once: with
+// this inlined wherever it was needed the kernel's code was 136 KB.
+__device__ __noinline__ void tc_share(const DecodeArgs& a, unsigned char* table, int c, TcShare* out)
+{
+    const SeqTable tab = seq_table_at(table, a);
+    const int NHl = a.B * a.Hkv;
+    const int R = slab_start(a, tab, NHl);
+    TcPart part;
+    part.R = R;
+    part.P = live_parts(R, a.nctas);
+    part.NHl = NHl;
+    part.scale = (float)part.P / (float)max(R, 1);
+    part.aligned = NHl * 4 <= a.nctas && R >= 4 * a.nctas;
+    // Only while no CTA would get more than 1.15 shares of rows (R / P), and every
+    // slab with rows gets a CTA of its own.
+#pragma unroll 1
+    for (int h = 0; h < NHl && part.aligned; ++h) {
+        const int rows = slab_start(a, tab, h + 1) - slab_start(a, tab, h);
+        const int n = part.cb(a, tab, h + 1) - part.cb(a, tab, h);
+        if (rows > 0 && (n < 1 || (float)rows * part.scale > 1.15f * (float)n)) part.aligned = false;
+    }
+    TcShare s = {0, 0, 0, 0, 0, 1, 0, 1};
+    if (c < part.P && R > 0) {
+        int next[2];
+#pragma unroll 1
+        for (int k = 0; k < 2; ++k) next[k] = part.start(a, tab, c + k);
+        s.A = next[0];
+        s.Bc = next[1];
+        int hs[2], c0[2], n[2];
+#pragma unroll 1
+        for (int k = 0; k < 2; ++k) {
+            hs[k] = slab_containing(a, tab, NHl, k ? s.Bc - 1 : s.A);
+            int c1;
+            n[k] = part.slab_ctas(a, tab, hs[k], slab_start(a, tab, hs[k]), slab_start(a, tab, hs[k] + 1), &c0[k], &c1);
+        }
+        s.hfirst = hs[0];
+        s.hlast = hs[1];
+        s.c0_first = c0[0];
+        s.n_first = n[0];
+        s.c0_last = c0[1];
+        s.n_last = n[1];
+    }
+    if ((threadIdx.x & 31) == 0) *out = s;
+}
+
+// Slabs with no rows belong to no CTA: their outputs are zero.
+template <int G>
+__device__ __noinline__ void write_empty_slabs_tc(const DecodeArgs& a, unsigned char* table, int lane)
+{
+    const SeqTable t = seq_table_at(table, a);
+#pragma unroll 1
+    for (int h = 0; h < a.B * a.Hkv; ++h)
+        if (slab_start(a, t, h) == slab_start(a, t, h + 1))
+#pragma unroll 1
+            for (int j = 0; j < a.NC; ++j)
+                write_out<G>(a, h / a.Hkv, h % a.Hkv, j, make_float4(0.f, 0.f, 0.f, 0.f), 0.f, lane);
+}
+
 template <int G>
 __global__ void __launch_bounds__(kTcThreads, 1)
     decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ CacheMaps maps)
@@ -436,9 +539,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     uint64_t* q_full = o_done + 2;                  // [2] Q buffer b holds the Q of its next segment
     uint64_t* fin = q_full + 2;                     // drain after a timeout
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + kOffTmem);
-    const SeqTable tab = seq_table_at(sm + kOffTable, a);
+    unsigned char* table = sm + kOffTable;
+    const SeqTable tab = seq_table_at(table, a);
+    const TcShare* share = reinterpret_cast<const TcShare*>(sm + kOffInfo);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
     const int NHl = a.B * a.Hkv;
     const int c = blockIdx.x;
 
@@ -457,33 +562,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __syncthreads();
     pdl_launch_dependents();
 
-    const int R = slab_start(a, tab, NHl);
+    if (warp == 0) tc_share(a, table, c, reinterpret_cast<TcShare*>(sm + kOffInfo));
+    __syncthreads();
     if (c == 0 && warp == 2) {
-        // Slabs with no rows belong to no CTA: their outputs are zero (after the
-        // wait, as every write of out).
-        pdl_wait();
-        for (int h = 0; h < NHl; ++h)
-            if (slab_start(a, tab, h) == slab_start(a, tab, h + 1))
-                for (int j = 0; j < a.NC; ++j)
-                    write_out<G>(a, h / a.Hkv, h % a.Hkv, j, make_float4(0.f, 0.f, 0.f, 0.f), 0.f, lane);
+        pdl_wait();  // as every write of out
+        write_empty_slabs_tc<G>(a, table, lane);
     }
-    TcPart part;
-    part.R = R;
-    part.P = live_parts(R, a.nctas);
-    part.NHl = NHl;
-    part.scale = (float)part.P / (float)max(R, 1);
-    part.aligned = NHl * 4 <= a.nctas && R >= 4 * a.nctas;
-    // Only while no CTA would get more than 1.15 shares of rows (R / P), and every
-    // slab with rows gets a CTA of its own.
-    for (int h = 0; h < NHl && part.aligned; ++h) {
-        const int rows = slab_start(a, tab, h + 1) - slab_start(a, tab, h);
-        const int n = part.cb(a, tab, h + 1) - part.cb(a, tab, h);
-        if (rows > 0 && (n < 1 || (float)rows * part.scale > 1.15f * (float)n)) part.aligned = false;
-    }
-    if (c >= part.P || R < 1) return;  // uniform: this CTA has no rows (no TMEM taken yet)
-    const int A = part.start(a, tab, c), Bc = part.start(a, tab, c + 1);
-    const int hfirst = slab_containing(a, tab, NHl, A);
-    const int hend = slab_containing(a, tab, NHl, Bc - 1) + 1;
+    const int A = uniform(share->A), Bc = uniform(share->Bc);
+    if (A >= Bc) return;  // uniform: this CTA has no rows (no TMEM taken yet)
+    const int hfirst = uniform(share->hfirst), hend = uniform(share->hlast) + 1;
+    int32_t* slot = reinterpret_cast<int32_t*>(sm + kOffSlots) + 6 * warp;
     const int NC = a.NC;
     const int NCpad = (NC + 15) & ~15;
     const float cs = a.qscale;
@@ -492,18 +580,21 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA
         // Starts at once (the copies need no TMEM); K and V of a tile go to their
-        // own rings, each issued as soon as its stage is free.
-        if (lane == 0) {
+        // own rings, each issued as soon as its stage is free. The whole warp runs the
+        // schedule, one lane issues.
+        {
+            const bool leads = elect_one();
             const uint64_t pol = evict_first_policy();
             TileWalk wk, wv;
-            wk.begin(a, tab, hfirst, hend, A, Bc);
+            wk.begin(a, table, hfirst, hend, A, Bc, slot);
             wv = wk;
             int tk = 0, tv = 0;
             bool waited = false;
             IdleBound idle;
-            while ((wk.more() || wv.more()) && !flags[kFlagAbort]) {
+#pragma unroll 1
+            while ((wk.more() || wv.more()) && !uniform(flags[kFlagAbort])) {
                 bool moved = false;
-                if (wk.more() && (tk < kKStages || test_phase(&k_empty[tk % kKStages], ((tk / kKStages) - 1) & 1))) {
+                if (wk.more() && (tk < kKStages || test_phase_warp(&k_empty[tk % kKStages], ((tk / kKStages) - 1) & 1))) {
                     if (tk == PRE && !waited) {
                         pdl_wait();  // later copies after the previous kernel, as in the other kernels
                         waited = true;
@@ -513,41 +604,49 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     // zeros past the end, so the copy stays in bounds either way).
                     in_bounds(row >= 0 && (a.rows_cap == 0 || row + wk.cnt() <= a.rows_cap), a.status);
                     const uint32_t bar = smem_u32(&k_full[s]), dst = smem_u32(ringK + s * kTcHalfTile);
-                    mbar_arrive_expect_tx(bar, kTcHalfTile);
+                    if (leads) {
+                        mbar_arrive_expect_tx(bar, kTcHalfTile);
 #pragma unroll
-                    for (int j = 0; j < kTcRows / kTcBoxRows; ++j) {
-                        tma_box(dst + j * kTcBoxRows * 128, &maps.k, 0, row + j * kTcBoxRows, bar, pol);
-                        tma_box(dst + kTcBox + j * kTcBoxRows * 128, &maps.k, 64, row + j * kTcBoxRows, bar, pol);
+                        for (int j = 0; j < kTcRows / kTcBoxRows; ++j) {
+                            tma_box(dst + j * kTcBoxRows * 128, &maps.k, 0, row + j * kTcBoxRows, bar, pol);
+                            tma_box(dst + kTcBox + j * kTcBoxRows * 128, &maps.k, 64, row + j * kTcBoxRows, bar, pol);
+                        }
                     }
                     ++tk;
-                    wk.next(a, tab);
+                    wk.next(a, table);
                     moved = true;
                 }
-                if (wv.more() && tv < tk && (tv < kVStages || test_phase(&v_empty[tv % kVStages], ((tv / kVStages) - 1) & 1))) {
+                if (wv.more() && tv < tk && (tv < kVStages || test_phase_warp(&v_empty[tv % kVStages], ((tv / kVStages) - 1) & 1))) {
                     const int s = tv % kVStages, row = wv.cache_row();
                     const uint32_t bar = smem_u32(&v_full[s]), dst = smem_u32(ringV + s * kTcHalfTile);
-                    mbar_arrive_expect_tx(bar, kTcHalfTile);
+                    if (leads) {
+                        mbar_arrive_expect_tx(bar, kTcHalfTile);
 #pragma unroll
-                    for (int j = 0; j < kTcRows / kTcBoxRows; ++j) {
-                        tma_box(dst + j * kTcBoxRows * 128, &maps.v, 0, row + j * kTcBoxRows, bar, pol);
-                        tma_box(dst + kTcBox + j * kTcBoxRows * 128, &maps.v, 64, row + j * kTcBoxRows, bar, pol);
+                        for (int j = 0; j < kTcRows / kTcBoxRows; ++j) {
+                            tma_box(dst + j * kTcBoxRows * 128, &maps.v, 0, row + j * kTcBoxRows, bar, pol);
+                            tma_box(dst + kTcBox + j * kTcBoxRows * 128, &maps.v, 64, row + j * kTcBoxRows, bar, pol);
+                        }
                     }
                     ++tv;
-                    wv.next(a, tab);
+                    wv.next(a, table);
                     moved = true;
                 }
                 if (moved) {
                     idle.progress();
-                } else if (idle.expired()) {
-                    atomicOr(a.status, kDevTmaTimeout);
-                    flags[kFlagAbort] = 1;
+                } else if (__any_sync(kFull, idle.expired())) {
+                    if (leads) {
+                        atomicOr(a.status, kDevTmaTimeout);
+                        flags[kFlagAbort] = 1;
+                    }
                     break;
                 } else {
                     __nanosleep(32);
                 }
             }
-            flags[kFlagKIssued] = tk;
-            flags[kFlagVIssued] = tv;
+            if (leads) {
+                flags[kFlagKIssued] = tk;
+                flags[kFlagVIssued] = tv;
+            }
         }
     } else {
         if (warp >= 2) {
@@ -555,10 +654,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // allocates TMEM: the first score product waits for both.
             const int st = tid - 64;
             pdl_wait();  // q and the outputs belong to the previous kernel's epoch
-            TileWalk w0;
-            w0.begin(a, tab, hfirst, hend, A, Bc);
-            const int h1 = later_segment_slab(w0.cu, a, tab, hend, A, Bc, 1);
-            load_q_tc<G>(a, w0.cu.h, sQ, st);
+            const int h1 = uniform(later_segment_slab(a, table, hfirst, hend, A, Bc, 1));
+            load_q_tc<G>(a, hfirst, sQ, st);
             if (h1 < hend) load_q_tc<G>(a, h1, sQ + kTcQBytes, st);
             fence_proxy_async_smem();
             named_sync(kBarSoft, kTcSoft);
@@ -575,7 +672,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tc_fence_before();
         named_sync(kBarTmem, kTcThreads - 32);
         tc_fence_after();
-        tmem = *tmem_slot;
+        tmem = (uint32_t)uniform((int)*tmem_slot);
     }
 
     if (warp == 1) {
@@ -583,8 +680,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         // Score products run up to kSBufs tiles ahead of the output products; a
         // score product needs its K stage, its S buffer free (the output product
         // of tile t - 4 issued, so its softmax is done) and, first in a segment,
-        // the segment's Q; an output product needs its P and its V stage.
-        if (lane == 0) {
+        // the segment's Q; an output product needs its P and its V stage. The whole
+        // warp runs the schedule on warp-uniform values and one lane issues: the
+        // products' operands are then uniform registers, which is what tcgen05.mma
+        // takes (a single-lane loop moved each of them there before each product:
+        // ~100 cycles a product instead of the pipe's 46 to 64).
+        {
+            const bool leads = elect_one();
             const uint32_t id1 = idesc(kTcQRows, kTcRows, 0, 0);
             const uint32_t id2 = idesc(128, 2 * NCpad, 1, 0);  // high and low parts of P side by side
             // Operand descriptors: every operand here has a stride byte offset of 1 KB,
@@ -600,7 +702,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const uint32_t dP = (uint32_t)sdesc(smem_u32(sP), 16, 1024);
             auto desc = [dhi](uint32_t lo) { return ((uint64_t)dhi << 32) | lo; };
             TileWalk w1;
-            w1.begin(a, tab, hfirst, hend, A, Bc);
+            w1.begin(a, table, hfirst, hend, A, Bc, slot);
             int t1 = 0, t2 = 0, seg = 0, seg_start = 0;
             int vs = 0;  // V stage of tile t2 (t2 % kVStages)
             // Bit t % kSBufs: tile t (between the two products) is one of the first two
@@ -609,6 +711,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             int qbuf = 0;  // Q buffer of the segment of tile t1
             bool issued = false, ok = true, qseen = false;
             IdleBound idle;
+#pragma unroll 1
             while (w1.more() || t2 < t1) {
                 bool moved = false;
                 // Output products first: the softmax group of tile t2 waits for it before
@@ -616,7 +719,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 // landed (the group's leader waits for it), so p_full is the one test.
                 if (t2 < t1) {
                     const int b = t2 & 1;
-                    if (test_phase(&p_full[b], (t2 >> 1) & 1)) {
+                    if (test_phase_warp(&p_full[b], (t2 >> 1) & 1)) {
                         tc_fence_after();
                         // O^T += V^T [P_hi P_lo] into the group's accumulator (the two
                         // halves are summed when O is read); a group's first tile of a
@@ -625,12 +728,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         const uint32_t pb = dP + (uint32_t)b * (kTcPBytes >> 4);
                         const uint32_t o = tmem + kTcOCol + b * kTcOCols;
                         const uint32_t fresh = (fresh_bits >> (t2 & (kSBufs - 1))) & 1u;
-                        umma(o, desc(va), desc(pb), id2, fresh ^ 1u);
+                        if (leads) {
+                            umma(o, desc(va), desc(pb), id2, fresh ^ 1u);
 #pragma unroll
-                        for (int k = 1; k < kTcRows / 16; ++k)
-                            umma(o, desc(va + k * (2048 >> 4)), desc(pb + k * (32 >> 4)), id2, 1u);
-                        umma_commit(smem_u32(&o_done[b]));
-                        umma_commit(smem_u32(&v_empty[vs]));
+                            for (int k = 1; k < kTcRows / 16; ++k)
+                                umma(o, desc(va + k * (2048 >> 4)), desc(pb + k * (32 >> 4)), id2, 1u);
+                            umma_commit(smem_u32(&o_done[b]));
+                            umma_commit(smem_u32(&v_empty[vs]));
+                        }
                         ++t2;
                         if (++vs == kVStages) vs = 0;
                         moved = true;
@@ -639,37 +744,39 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 if (w1.more() && t1 < t2 + kSBufs) {
                     const int s = t1 & (kKStages - 1);
                     const bool first = w1.first();
-                    if (first && !qseen && test_phase(&q_full[seg & 1], (seg >> 1) & 1)) {
+                    if (first && !qseen && test_phase_warp(&q_full[seg & 1], (seg >> 1) & 1)) {
                         qbuf = seg & 1;
                         ++seg;
                         seg_start = t1;
                         qseen = true;  // this segment's Q is in place
                     }
-                    if ((!first || qseen) && test_phase(&k_full[s], (t1 / kKStages) & 1)) {
+                    if ((!first || qseen) && test_phase_warp(&k_full[s], (t1 / kKStages) & 1)) {
                         tc_fence_after();
                         // S^T[64 x 64] = Q[64 x 128] K^T: k-steps of 16 dims (+32 B inside a
                         // 64-dim half, +kTcBox or +kTcQHalf to the next half).
                         const uint32_t qa = dQ + (uint32_t)qbuf * (kTcQBytes >> 4);
                         const uint32_t kb = dK + (uint32_t)s * (kTcHalfTile >> 4);
                         const uint32_t d = tmem + (t1 & (kSBufs - 1)) * kTcRows;
+                        if (leads) {
 #pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            umma(d, desc(qa + (k >> 2) * (kTcQHalf >> 4) + (k & 3) * 2),
-                                 desc(kb + (k >> 2) * (kTcBox >> 4) + (k & 3) * 2), id1, k > 0 ? 1u : 0u);
-                        umma_commit(smem_u32(&s_full[t1 & (kSBufs - 1)]));
-                        umma_commit(smem_u32(&k_empty[s]));
+                            for (int k = 0; k < 8; ++k)
+                                umma(d, desc(qa + (k >> 2) * (kTcQHalf >> 4) + (k & 3) * 2),
+                                     desc(kb + (k >> 2) * (kTcBox >> 4) + (k & 3) * 2), id1, k > 0 ? 1u : 0u);
+                            umma_commit(smem_u32(&s_full[t1 & (kSBufs - 1)]));
+                            umma_commit(smem_u32(&k_empty[s]));
+                        }
                         const uint32_t bit = 1u << (t1 & (kSBufs - 1));
                         fresh_bits = (t1 - seg_start < 2) ? (fresh_bits | bit) : (fresh_bits & ~bit);
                         issued = true;
                         qseen = false;
                         ++t1;
-                        w1.next(a, tab);
+                        w1.next(a, table);
                         moved = true;
                     }
                 }
                 if (moved) {
                     idle.progress();
-                } else if (flags[kFlagAbort] || idle.expired()) {
+                } else if (uniform(flags[kFlagAbort]) || __any_sync(kFull, idle.expired())) {
                     // Another role gave up, or nothing moved within the bound.
                     ok = false;
                     break;
@@ -677,11 +784,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     __nanosleep(20);
                 }
             }
-            if (!ok) {
-                atomicOr(a.status, kDevTmaTimeout);
-                flags[kFlagAbort] = 1;
+            if (leads) {
+                if (!ok) {
+                    atomicOr(a.status, kDevTmaTimeout);
+                    flags[kFlagAbort] = 1;
+                }
+                flags[kFlagMmaLast] = issued ? 1 : 0;
             }
-            flags[kFlagMmaLast] = issued ? 1 : 0;
+            __syncwarp();
         }
     } else if (warp >= 2) {
         // ---------------------------------------------------------------- softmax groups and epilogue
@@ -698,7 +808,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const int dim = 32 * quarter + lane;
         const uint32_t my_o = tmem + lane_addr + kTcOCol + gi * kTcOCols;
         TileWalk w;
-        w.begin(a, tab, hfirst, hend, A, Bc);
+        w.begin(a, table, hfirst, hend, A, Bc, slot);
         int seg_idx = -1;              // index of the current segment
         float m = -INFINITY, l = 0.f;  // this group's running max (log2 units) and sum of column col
         int t = 0, seg_start = 0;
@@ -706,7 +816,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         bool stop = false;             // set at a segment's end, the same in both groups
         // After a wait runs out a group keeps walking the tiles (without work) so that
         // both groups meet at every segment's end: a named barrier has no bound.
-        for (; w.more() && !stop; ++t, w.next(a, tab)) {
+#pragma unroll 1
+        for (; w.more() && !stop; ++t, w.next(a, table)) {
             if (w.first()) {
                 seg_start = t;
                 ++seg_idx;
@@ -738,7 +849,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     tc_fence_before();
                 }
                 named_sync(gbar, kTcGroup);
-                if (!flags[kFlagOk + gi]) {
+                if (!uniform(flags[kFlagOk + gi])) {
                     named_sync(gbar, kTcGroup);  // the flag is rewritten at the group's next tile
                 } else {
                     tc_fence_after();
@@ -775,10 +886,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                             tc_fence_before();
                         }
                         named_sync(gbar, kTcGroup);
-                        go = flags[kFlagOk2 + gi];
+                        go = uniform(flags[kFlagOk2 + gi]) != 0;
                         tc_fence_after();
-                        const bool rescale = flags[kFlagVote + 4 * gi] | flags[kFlagVote + 4 * gi + 1] |
-                                             flags[kFlagVote + 4 * gi + 2] | flags[kFlagVote + 4 * gi + 3];
+                        const bool rescale = uniform(flags[kFlagVote + 4 * gi] | flags[kFlagVote + 4 * gi + 1] |
+                                                     flags[kFlagVote + 4 * gi + 2] | flags[kFlagVote + 4 * gi + 3]) != 0;
                         if (go && rescale) {
                             float alpha = 1.f;
                             if (vote) {
@@ -851,12 +962,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // the two groups' states, and this segment's output or partial.
             if (leader) flags[kFlagSegOk] = !flags[kFlagAbort];
             named_sync(kBarSoft, kTcSoft);  // every S product of the segment was seen done by its group
-            const bool seg_ok = flags[kFlagSegOk];
-            const int h = w.cu.h, p0h = w.cu.p0, p1h = w.cu.p0 + w.cu.n_h;
-            const bool whole = w.cu.s0 == p0h && w.cu.s1 == p1h;
+            const bool seg_ok = uniform(flags[kFlagSegOk]) != 0;
+            const int h = w.sg.h;
+            const bool whole = w.rows == w.sg.p1 - w.sg.p0;
             // Q of the segment after next into this segment's buffer (its score
             // products are all done: each group saw its tiles' S).
-            const int h2 = later_segment_slab(w.cu, a, tab, hend, A, Bc, 2);
+            const int h2 = uniform(later_segment_slab(a, table, h, hend, A, Bc, 2));
             if (h2 < hend) {
                 load_q_tc<G>(a, h2, sQ + (seg_idx & 1) * kTcQBytes, st);
                 fence_proxy_async_smem();
@@ -881,7 +992,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 tc_fence_before();
             }
             named_sync(kBarSoft, kTcSoft);
-            const bool merge_ok = flags[kFlagOk] && flags[kFlagOk + 1];
+            const bool merge_ok = uniform(flags[kFlagOk] && flags[kFlagOk + 1]) != 0;
             stop = !merge_ok;
             tc_fence_after();
             // Merge of the groups: group gi writes the columns 32 gi .. 32 gi + 31 of every dimension.
@@ -953,9 +1064,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         for (int e = 0; e < 2; ++e) {
             const int h = e == 0 ? hfirst : hend - 1;
             if (e == 1 && h == hfirst) break;
-            const int p0 = slab_start(a, tab, h), p1 = slab_start(a, tab, h + 1);
-            int c0 = 0, c1 = 0;
-            const int nct = part.slab_ctas(a, tab, h, p0, p1, &c0, &c1);
+            const int c0 = uniform(e == 0 ? share->c0_first : share->c0_last);
+            const int nct = uniform(e == 0 ? share->n_first : share->n_last), c1 = c0 + nct - 1;
             if (nct <= 1) continue;  // uniform: written at its segment's end
             int32_t* ctr = a.slab_count + (int64_t)h * kMaxCols * 2;
             if (leader) {
@@ -979,7 +1089,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 flags[kFlagSegOk] = ok;
             }
             named_sync(kBarSoft, kTcSoft);
-            if (flags[kFlagSegOk]) {
+            if (uniform(flags[kFlagSegOk])) {
                 const int k = c - c0;  // rank of this CTA among the slab's CTAs
                 const int j0 = (int)((int64_t)k * NC / nct), j1 = (int)((int64_t)(k + 1) * NC / nct);
                 const int hb = h / a.Hkv, hg = h - hb * a.Hkv;
@@ -1064,9 +1174,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             for (int u = max(0, nk - kKStages); u < nk; ++u) wait_phase(&k_full[u % kKStages], (u / kKStages) & 1);
             for (int u = max(0, nv - kVStages); u < nv; ++u) wait_phase(&v_full[u % kVStages], (u / kVStages) & 1);
         }
-        if (tid == 32 && flags[kFlagMmaLast]) {
-            umma_commit(smem_u32(fin));
-            wait_phase(fin, 0);
+        if (warp == 1 && uniform(flags[kFlagMmaLast])) {
+            if (elect_one()) {
+                umma_commit(smem_u32(fin));
+                wait_phase(fin, 0);
+            }
+            __syncwarp();
         }
         tc_fence_before();
         __syncthreads();
