@@ -423,7 +423,10 @@ __global__ void __launch_bounds__(MKFor<G, NT, MULTI>::NW * 32, 1)
     constexpr int NCC = MULTI ? 0 : G;
     const int NC = MULTI ? a.NC : G;
     constexpr int TR = C::TR, NS = C::NS, NW = C::NW;
-    constexpr int NPRE = 2;  // half-tiles fetched before the wait for the previous kernel (more compete with its merge)
+    // Half-tiles fetched before the wait for the previous kernel: they compete with its
+    // merge, and fill the memory pipe while it runs (us per step with 2, 3, 4: 128K
+    // 1,018 / 1,007 / 1,033, 32K 425 / 423 / 461, ragged batch of 16 662 / 655 / 656).
+    constexpr int NPRE = NS < 3 ? NS : 3;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // The ring starts on a 1024-byte boundary (the swizzle pattern's period).
     unsigned char* smem = smem_raw + ((C::kAlign - (smem_u32(smem_raw) & (C::kAlign - 1))) & (C::kAlign - 1));
