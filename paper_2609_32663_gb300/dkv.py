@@ -159,7 +159,9 @@ def _dev(t, name, dtypes=None, numel=None, min_numel=None):
     addresses, so it is refused before the call."""
     if t is None or isinstance(t, int):
         return t
-    why = None
+    if (getattr(t, "is_cuda", False) and t.is_contiguous() and (dtypes is None or t.dtype in dtypes)
+            and (numel is None or t.numel() == numel) and (min_numel is None or t.numel() >= min_numel)):
+        return t.data_ptr()
     if not getattr(t, "is_cuda", False):
         why = "must be a CUDA tensor"
     elif not t.is_contiguous():
@@ -168,34 +170,57 @@ def _dev(t, name, dtypes=None, numel=None, min_numel=None):
         why = f"has dtype {t.dtype}, expected one of {dtypes}"
     elif numel is not None and t.numel() != numel:
         why = f"has {t.numel()} elements, expected {numel}"
-    elif min_numel is not None and t.numel() < min_numel:
+    else:
         why = f"has {t.numel()} elements, needs at least {min_numel}"
-    if why:
-        raise DkvError(DKV_ERR_INVALID_ARG, "argument check", f"{name} {why}")
-    return t.data_ptr()
+    raise DkvError(DKV_ERR_INVALID_ARG, "argument check", f"{name} {why}")
+
+
+# Element types of the buffer arguments, and torch's own lookup of the current
+# stream: resolved once, on the first call that takes tensors (the binding can be
+# imported without torch). Per call these were a third of the binding's time.
+_T = None
+
+
+class _Torch:
+    def __init__(self):
+        import torch
+        self.torch = torch
+        self.bf16 = (torch.bfloat16, torch.int16)
+        self.i32 = (torch.int32,)
+        self.f32 = (torch.float32,)
+        self.u8 = (torch.uint8,)
+        C = torch._C
+        self.raw_stream = getattr(C, "_cuda_getCurrentRawStream", None)
+        self.device = getattr(C, "_cuda_getDevice", None)
+
+
+def _torch():
+    global _T
+    if _T is None:
+        _T = _Torch()
+    return _T
 
 
 def _bf16():
-    import torch
-    return (torch.bfloat16, torch.int16)
+    return _torch().bf16
 
 
 def _i32():
-    import torch
-    return (torch.int32,)
+    return _torch().i32
 
 
 def _f32():
-    import torch
-    return (torch.float32,)
+    return _torch().f32
 
 
 def _stream(stream):
     if stream is None:
-        import torch
-        if not torch.cuda.is_available():
+        t = _torch()
+        if t.raw_stream is not None and t.torch.cuda.is_initialized():
+            return t.raw_stream(t.device())
+        if not t.torch.cuda.is_available():
             return None
-        return torch.cuda.current_stream().cuda_stream
+        return t.torch.cuda.current_stream().cuda_stream
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
@@ -207,6 +232,7 @@ class Plan:
         self.shape = shape
         self.B = B
         self.dense = dense
+        self._info = None  # dkv_plan_query's answer: a plan's sizes and addresses never change
 
     def close(self):
         if self.handle:
@@ -220,10 +246,14 @@ class Plan:
             pass
 
     @property
-    def _as_parameter_(self):
+    def address(self) -> int:
         if not self.handle:
             raise ValueError("plan already freed")
-        return ctypes.c_void_p(self.handle)
+        return self.handle
+
+    @property
+    def _as_parameter_(self):
+        return ctypes.c_void_p(self.address)
 
 
 def dkv_map_pattern(M, ctx_len, shape: Shape, reserve_rows: int = 0, stream=None) -> Plan:
@@ -328,7 +358,8 @@ def dkv_plan_query(plan: Plan) -> PlanInfo:
     pl, po, pi, px = (ctypes.c_void_p() for _ in range(4))
     _check(lib().dkv_plan_query(plan, ctypes.byref(tr), ctypes.byref(kr), ctypes.byref(pl),
                                 ctypes.byref(po), ctypes.byref(pi), ctypes.byref(px)), "dkv_plan_query")
-    return PlanInfo(tr.value, kr.value, pl.value, po.value, pi.value, px.value)
+    plan._info = PlanInfo(tr.value, kr.value, pl.value, po.value, pi.value, px.value)
+    return plan._info
 
 
 def dkv_compact(plan: Plan, K, V, Kc, Vc, T_stride: int | None = None, stream=None):
@@ -343,21 +374,22 @@ def dkv_compact(plan: Plan, K, V, Kc, Vc, T_stride: int | None = None, stream=No
 
 
 def _decode_ptrs(plan: Plan, q, k_new, v_new, n_appended, Kc, Vc, Q: int = 1):
-    sh, B = plan.shape, plan.B
-    rows = dkv_plan_query(plan).total_rows * 128
-    return (_dev(q, "q", _bf16(), numel=B * Q * sh.H * 128),
-            _dev(k_new, "k_new", _bf16(), numel=B * sh.H_kv * 128),
-            _dev(v_new, "v_new", _bf16(), numel=B * sh.H_kv * 128),
-            _dev(n_appended, "n_appended", _i32(), numel=B),
-            _dev(Kc, "Kc", _bf16(), min_numel=rows), _dev(Vc, "Vc", _bf16(), min_numel=rows))
+    sh, B, T = plan.shape, plan.B, _torch()
+    plan.address  # a freed plan is refused before its sizes are used
+    rows = (plan._info or dkv_plan_query(plan)).total_rows * 128
+    return (_dev(q, "q", T.bf16, B * Q * sh.H * 128),
+            _dev(k_new, "k_new", T.bf16, B * sh.H_kv * 128),
+            _dev(v_new, "v_new", T.bf16, B * sh.H_kv * 128),
+            _dev(n_appended, "n_appended", T.i32, B),
+            _dev(Kc, "Kc", T.bf16, None, rows), _dev(Vc, "Vc", T.bf16, None, rows))
 
 
 def dkv_decode_attn(plan: Plan, layer: int, q, k_new, v_new, n_appended, Kc, Vc, out, scale: float = 0.0,
                     stream=None):
     qp, kp, vp, np_, kc, vc = _decode_ptrs(plan, q, k_new, v_new, n_appended, Kc, Vc)
     op = _dev(out, "out", _f32(), numel=plan.B * plan.shape.H * 128)
-    _check(lib().dkv_decode_attn(plan, int(layer), qp, kp, vp, np_, kc, vc, ctypes.c_float(scale), op,
-                                 _stream(stream)), "dkv_decode_attn")
+    _check(lib().dkv_decode_attn(plan.address, int(layer), qp, kp, vp, np_, kc, vc, scale, op, _stream(stream)),
+           "dkv_decode_attn")
 
 
 def dkv_decode_multi(plan: Plan, layer: int, q, num_queries: int, n_appended, Kc, Vc, out, scale: float = 0.0,
@@ -367,7 +399,7 @@ def dkv_decode_multi(plan: Plan, layer: int, q, num_queries: int, n_appended, Kc
     Q = max(int(num_queries), 1)
     qp, _, _, np_, kc, vc = _decode_ptrs(plan, q, None, None, n_appended, Kc, Vc, Q=Q)
     op = _dev(out, "out", _f32(), numel=plan.B * Q * plan.shape.H * 128)
-    _check(lib().dkv_decode_multi(plan, int(layer), qp, int(num_queries), np_, kc, vc, ctypes.c_float(scale), op,
+    _check(lib().dkv_decode_multi(plan.address, int(layer), qp, int(num_queries), np_, kc, vc, scale, op,
                                   _stream(stream)), "dkv_decode_multi")
 
 
@@ -427,13 +459,13 @@ def dkv_decode_attn_noalloc(shape: Shape, B: int, layer: int, reserve_rows: int,
                             v_new, n_appended, Kc, Vc, out, scale: float = 0.0, status=None, stream=None):
     """Decode attention that allocates no device memory; d_len/d_off/d_ioff are
     device addresses (ints) or tensors of the plan metadata."""
-    sh = shape.c()
+    T = _torch()
     _check(lib().dkv_decode_attn_noalloc(
-        ctypes.byref(sh), int(B), int(layer), int(reserve_rows), _dev(d_len, "d_len"), _dev(d_off, "d_off"),
-        _dev(d_ioff, "d_ioff"), _dev(q, "q", _bf16(), numel=B * shape.H * 128),
-        _dev(k_new, "k_new", _bf16(), numel=B * shape.H_kv * 128), _dev(v_new, "v_new", _bf16(), numel=B * shape.H_kv * 128),
-        _dev(n_appended, "n_appended", _i32(), numel=B), _dev(Kc, "Kc", _bf16()), _dev(Vc, "Vc", _bf16()),
-        ctypes.c_float(scale), _dev(out, "out", _f32(), numel=B * shape.H * 128), _dev(status, "status", _i32()),
+        ctypes.byref(shape.c()), int(B), int(layer), int(reserve_rows), _dev(d_len, "d_len"), _dev(d_off, "d_off"),
+        _dev(d_ioff, "d_ioff"), _dev(q, "q", T.bf16, B * shape.H * 128),
+        _dev(k_new, "k_new", T.bf16, B * shape.H_kv * 128), _dev(v_new, "v_new", T.bf16, B * shape.H_kv * 128),
+        _dev(n_appended, "n_appended", T.i32, B), _dev(Kc, "Kc", T.bf16), _dev(Vc, "Vc", T.bf16),
+        scale, _dev(out, "out", _f32(), numel=B * shape.H * 128), _dev(status, "status", _i32()),
         _stream(stream)), "dkv_decode_attn_noalloc")
 
 
