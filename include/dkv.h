@@ -271,12 +271,9 @@ dkv_status dkv_decode_attn(const dkv_plan* plan, int32_t layer, const void* q,
  * all queries:
  *   <= 16 columns  a split-K kernel whose warps multiply 16-row tiles on the
  *                  warp-level tensor-core path, then a combine kernel;
- *   17..64         one tcgen05 kernel: 64-row tiles staged by TMA, scores and
- *                  outputs accumulated in tensor memory, and the CTAs that
- *                  share a slab merge their partials inside the same launch.
- *                  It is a cooperative launch (all CTAs resident at once), so
- *                  it fails with DKV_ERR_CUDA where the device cannot grant
- *                  one (for example under a partitioned device).
+ *   17..64         a tcgen05 kernel: 64-row tiles staged by TMA, scores and
+ *                  outputs accumulated in tensor memory; then a combine kernel
+ *                  merges the slabs that several CTAs share.
  * Other arguments, ordering and errors are those of dkv_decode_attn; a
  * num_queries * G above 64 is DKV_ERR_INVALID_ARG.
  */

@@ -34,7 +34,7 @@ struct dkv_plan {
     float* d_work = nullptr;    // split-K partials
     float* d_exch = nullptr;    // exchange of the fused merge: slots x kMaxCols x (128 + 2) words, 0 between launches
     int64_t exch_slots = 0;     // (CTA, slab) slots of the exchange
-    int32_t* d_slab_count = nullptr;  // [B*H_kv][cols][2] arrival / done counters of the tcgen05 kernel's merge
+    int32_t* d_slab_parts = nullptr;  // [B*H_kv][2] which CTAs hold a slab's partials (tcgen05 kernel)
     dkv::DecodeConfig cfg{};         // the decode step's kernel (cfg_f32 or cfg_mma)
     dkv::DecodeConfig cfg_f32{};     // fp32 kernel (caches of 2^31 rows or more)
     dkv::DecodeConfig cfg_mma{};     // tensor-core kernel of the decode step
@@ -42,7 +42,6 @@ struct dkv_plan {
     dkv::DecodeConfig cfg_multi{};   // multi-query, two column tiles (tensor-core plans)
     dkv::DecodeConfig cfg_tc{};      // multi-query, 17 to 64 columns on tcgen05 (tensor-core plans)
     dkv::WorkspaceLayout work{};     // carve-up of d_work
-    int cols_cap = 0;                // columns the workspace and counters are sized for
     int use_mma = 0;  // tensor-core decode kernel (needs the cache's row count for its tensor maps)
     int64_t inplace_stride = 0;  // > 0: slab h lives at rows h * stride of the dense buffer (in place)
     int32_t* d_order = nullptr;  // in place: [NH] slabs by length, longest first, then a claim counter
@@ -180,7 +179,6 @@ dkv_status plan_configs(dkv_plan* p)
         ctas = std::max<int64_t>(ctas, c->nctas);
         warp_records = std::max<int64_t>(warp_records, (int64_t)c->nctas * c->nwarps);
     }
-    p->cols_cap = dkv::kMaxCols;
     const int64_t NHl = (int64_t)p->B * p->s.H_kv;
     p->work = dkv::workspace_layout(ctas + NHl, dkv::kTcMaxCols, warp_records, dkv::kMaxCols);
     p->exch_slots = ctas + NHl;
@@ -198,7 +196,7 @@ struct ZeroBlock {
 ZeroBlock take_zeroed(ArenaLayout& lay, const dkv_plan* p, size_t extra)
 {
     ZeroBlock z;
-    z.count = 1 + (size_t)2 * p->B * p->s.H_kv * p->cols_cap + extra;
+    z.count = 2 + (size_t)2 * p->B * p->s.H_kv + extra;
     z.off = lay.take<int32_t>(z.count);
     return z;
 }
@@ -206,7 +204,7 @@ ZeroBlock take_zeroed(ArenaLayout& lay, const dkv_plan* p, size_t extra)
 void place_zeroed(dkv_plan* p, const ZeroBlock& z)
 {
     p->d_status = at<int32_t>(p->d_arena, z.off);
-    p->d_slab_count = p->d_status + 1;
+    p->d_slab_parts = p->d_status + 2;  // 8-byte aligned
 }
 
 // The decode kernel of a plan whose row count is known.
@@ -298,7 +296,6 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
         release(p);
         return e;
     };
-    p->cols_cap = dkv::kMaxCols;
 
     ArenaLayout lay;
     const size_t o_len = lay.take<int32_t>((size_t)NH), o_off = lay.take<int64_t>((size_t)NH + 1),
@@ -628,7 +625,7 @@ dkv_status decode_args(const dkv_plan* p, int32_t layer, const void* q, const vo
     a->exch_o = p->d_exch;
     a->exch_ml = p->d_exch + p->exch_slots * dkv::kMaxCols * dkv::kHeadDim;
     a->out = out;
-    a->slab_count = p->d_slab_count;
+    a->slab_parts = p->d_slab_parts;
     a->merge_extra = fault("merge") ? 1 : 0;
     a->status = p->d_status;
     a->rows_cap = p->total_rows;

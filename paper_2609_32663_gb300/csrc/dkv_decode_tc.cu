@@ -4,8 +4,7 @@
 // (queries x heads of a KV head's group) per slab.
 //
 // Work split: the layer's rows (every slab end to end, plus the rows appended in
-// earlier steps) are cut into contiguous CTA ranges (one CTA per SM, a
-// cooperative launch, so every CTA is resident at once): whole numbers of CTAs
+// earlier steps) are cut into contiguous CTA ranges (one CTA per SM): whole numbers of CTAs
 // per slab while the slabs are few (TcPart below), else equal ranges as in the
 // other decode kernels. A CTA walks its range in tiles of 64 rows, slab segment
 // by slab segment (a segment: the part of one slab inside the CTA's range).
@@ -47,25 +46,27 @@
 // the score products run on across a slab boundary.
 //
 // A slab wholly inside one CTA is written out at its segment's end. Otherwise
-// each CTA of the slab writes its partial (m, l, o of every column) and counts
-// itself in; once the CTA's range is done it waits (bounded) until all the
-// slab's CTAs have counted in, then merges its share of the slab's columns
-// (CTA k of the slab's nct CTAs takes columns k NC / nct .. (k+1) NC / nct):
-// the merge is spread over the slab's CTAs instead of falling on the last one.
-//
-// What bounds it: a 64-row tile is 32 KB, 0.73 us at an SM's share of HBM, and its
-// products need 0.3 us of the tensor pipe's operand bandwidth, so the schedules of
-// the roles set the pace. They run on warp-uniform values (uniform()): with a
-// single-lane MMA loop every operand went through a vector register and a move
-// before each product, and the kernel's code was 136 KB of walkers and partition
-// arithmetic, repeated inline, now 93. Same box, 4 layers at 128K: 64 columns 236
-// -> 189 us, 32 columns 229 -> 173; Qwen shape 64K x 4, 28 columns 250 -> 180.
+// each CTA of the slab writes its partial (m, l, o of every column) and a second
+// kernel combines them, one warp a (slab, column). Both launches are ordinary ones
+// that overlap their start with the end of the previous kernel. (Merging inside
+// this kernel needed every CTA resident, so a cooperative launch, which starts
+// only after the previous kernel has drained: 2.5 us, then 4 us of prologue and 5
+// us of waiting for the slab's slowest CTA. 4 layers at 128K: 64 columns 189 ->
+// 172 us, 32 columns 170 -> 152; 32K, 8 layers, 64 columns 757 -> 615.)
 //
 // Every wait is bounded (polls and 2 s). A wait that runs out sets a
 // DKV_DEV_* bit, the roles stop (the softmax groups keep walking the tiles,
 // without work, so that they still meet at every named barrier), the copies and
 // products in flight are drained with the same bound, and TMEM is freed before
 // the CTA exits.
+//
+// What bounds it: a 64-row tile is 32 KB, 0.73 us at an SM's share of HBM, and its
+// products need 0.3 us of the tensor pipe's operand bandwidth, so the schedules of
+// the roles set the pace. They run on warp-uniform values (uniform()): with a
+// single-lane MMA loop every operand went through a vector register and a move
+// before each product, and the kernel's code was 136 KB of walkers and partition
+// arithmetic, repeated inline, now 75. Same box, 4 layers at 128K: 64 columns 236
+// -> 189 us, 32 columns 229 -> 173; Qwen shape 64K x 4, 28 columns 250 -> 180.
 #include "dkv_decode_common.cuh"
 
 #include <cuda.h>
@@ -88,6 +89,7 @@ constexpr int kTcQRows = 64;                   // M of the score product: the mo
 constexpr int kTcQHalf = kTcQRows * 128;       // one 64-dim half of Q (8 KB)
 constexpr int kTcQBytes = 2 * kTcQHalf;        // Q as the A operand: 64 rows x 128 dims (two buffers: segments alternate)
 constexpr int kTcPBytes = 2 * kTcMaxCols * 128;  // one P buffer: high parts (rows 0..NCpad-1), then low parts, 64 rows each
+constexpr int kTcPre = 1;                      // tiles a CTA fetches before waiting for the previous kernel
 constexpr int kSBufs = 4;                      // TMEM score buffers
 static_assert((kKStages & (kKStages - 1)) == 0 && (kSBufs & (kSBufs - 1)) == 0, "indexed by masks");
 constexpr int kTcTmemCols = 512;               // S buffers at columns 0, 64, 128, 192; O of group g at 256 + 128 g
@@ -132,7 +134,7 @@ constexpr int kNumFlags = 24;
 constexpr float kSlackTc = 32.f;
 
 // Device status bits (include/dkv.h).
-constexpr int kDevTmaTimeout = 0x2, kDevMergeTimeout = 0x4;
+constexpr int kDevTmaTimeout = 0x2;
 
 // ------------------------------------------------------------ tcgen05 wrappers
 // Shared-memory matrix descriptor: start address, leading and stride byte
@@ -313,6 +315,7 @@ struct TileWalk {
     Segment sg;       // `left` and `row` run on tile by tile
     int hend, A, B;
     int rows;         // of the whole segment
+    bool rows_from_start;  // the segment begins with its slab's first row
     int32_t* slot;    // the warp's segment slot in shared memory
     __device__ __forceinline__ void begin(const DecodeArgs& a, unsigned char* table, int hfirst, int hend_, int A_, int B_,
                                           int32_t* slot_)
@@ -328,6 +331,7 @@ struct TileWalk {
         find_segment(a, table, h, hend, A, B, slot);
         sg = read_segment(slot);
         rows = sg.left;
+        rows_from_start = max(A, sg.p0) == sg.p0;
     }
     __device__ __forceinline__ bool more() const { return sg.left > 0; }
     __device__ __forceinline__ int cnt() const { return min(kTcRows, sg.left); }
@@ -360,15 +364,21 @@ template <int G>
 __device__ void load_q_tc(const DecodeArgs& a, int h, unsigned char* sQ, int tid)
 {
     const int b = h / a.Hkv, g = h - b * a.Hkv;
-    for (int i = tid; i < kTcQRows * 16; i += kTcSoft) {
-        const int c = i >> 4, ch = i & 15;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    constexpr int kPer = kTcQRows * 16 / kTcSoft;
+    uint4 v[kPer];  // every load before the first store: one round trip
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int i = tid + u * kTcSoft, c = i >> 4, ch = i & 15;
+        v[u] = make_uint4(0u, 0u, 0u, 0u);
         if (c < a.NC) {
             const int qi = c / G, j = c - qi * G;
-            const uint4* src = reinterpret_cast<const uint4*>(a.q + (((int64_t)b * a.Q + qi) * a.H + g * G + j) * kHeadDim);
-            v = __ldg(src + ch);
+            v[u] = __ldg(reinterpret_cast<const uint4*>(a.q + (((int64_t)b * a.Q + qi) * a.H + g * G + j) * kHeadDim) + ch);
         }
-        *reinterpret_cast<uint4*>(sQ + (ch >> 3) * kTcQHalf + sw128(c, ch & 7)) = v;
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int i = tid + u * kTcSoft, c = i >> 4, ch = i & 15;
+        *reinterpret_cast<uint4*>(sQ + (ch >> 3) * kTcQHalf + sw128(c, ch & 7)) = v[u];
     }
 }
 
@@ -449,18 +459,16 @@ struct TcPart {
     }
 };
 
-// A CTA's share of the layer: its rows [A, Bc), first and last slab, and for both
-// the CTAs they lie in (their first, and their count).
+// A CTA's share of the layer: its rows [A, Bc), first and last slab, and in how many
+// CTAs these two lie.
 struct TcShare {
-    int A, Bc, hfirst, hlast, c0_first, n_first, c0_last, n_last;
+    int A, Bc, hfirst, hlast, n_first, n_last;
 };
-static_assert(sizeof(TcShare) == kInfoWords * 4, "the info words");
+static_assert(sizeof(TcShare) <= kInfoWords * 4, "the info words");
 
-// One warp computes it for the CTA (A = Bc: no rows). Out of line and once: with
-// this inlined wherever it was needed the kernel's code was 136 KB.
-__device__ __noinline__ void tc_share(const DecodeArgs& a, unsigned char* table, int c, TcShare* out)
+// The layer's partition (one warp).
+__device__ __forceinline__ TcPart tc_partition(const DecodeArgs& a, const SeqTable& tab)
 {
-    const SeqTable tab = seq_table_at(table, a);
     const int NHl = a.B * a.Hkv;
     const int R = slab_start(a, tab, NHl);
     TcPart part;
@@ -471,34 +479,47 @@ __device__ __noinline__ void tc_share(const DecodeArgs& a, unsigned char* table,
     part.aligned = NHl * 4 <= a.nctas && R >= 4 * a.nctas;
     // Only while no CTA would get more than 1.15 shares of rows (R / P), and every
     // slab with rows gets a CTA of its own.
+    bool uneven = false;
+    if (part.aligned) {
 #pragma unroll 1
-    for (int h = 0; h < NHl && part.aligned; ++h) {
-        const int rows = slab_start(a, tab, h + 1) - slab_start(a, tab, h);
-        const int n = part.cb(a, tab, h + 1) - part.cb(a, tab, h);
-        if (rows > 0 && (n < 1 || (float)rows * part.scale > 1.15f * (float)n)) part.aligned = false;
-    }
-    TcShare s = {0, 0, 0, 0, 0, 1, 0, 1};
-    if (c < part.P && R > 0) {
-        int next[2];
-#pragma unroll 1
-        for (int k = 0; k < 2; ++k) next[k] = part.start(a, tab, c + k);
-        s.A = next[0];
-        s.Bc = next[1];
-        int hs[2], c0[2], n[2];
-#pragma unroll 1
-        for (int k = 0; k < 2; ++k) {
-            hs[k] = slab_containing(a, tab, NHl, k ? s.Bc - 1 : s.A);
-            int c1;
-            n[k] = part.slab_ctas(a, tab, hs[k], slab_start(a, tab, hs[k]), slab_start(a, tab, hs[k] + 1), &c0[k], &c1);
+        for (int h = threadIdx.x & 31; h < NHl; h += 32) {
+            const int rows = slab_start(a, tab, h + 1) - slab_start(a, tab, h);
+            const int n = part.cb(a, tab, h + 1) - part.cb(a, tab, h);
+            uneven |= rows > 0 && (n < 1 || (float)rows * part.scale > 1.15f * (float)n);
         }
-        s.hfirst = hs[0];
-        s.hlast = hs[1];
-        s.c0_first = c0[0];
-        s.n_first = n[0];
-        s.c0_last = c0[1];
-        s.n_last = n[1];
     }
-    if ((threadIdx.x & 31) == 0) *out = s;
+    if (__any_sync(kFull, uneven)) part.aligned = false;
+    return part;
+}
+
+// One warp computes the CTA's share (A = Bc: no rows). Out of line and once: with
+// this inlined wherever it was needed the kernel's code was 136 KB.
+__device__ __noinline__ void tc_share(const DecodeArgs& a, unsigned char* table, int c, TcShare* out)
+{
+    const SeqTable tab = seq_table_at(table, a);
+    const TcPart part = tc_partition(a, tab);
+    const int NHl = part.NHl, R = part.R, lane = threadIdx.x & 31;
+    if (c >= part.P || R < 1) {
+        if (lane == 0) *out = TcShare{0, 0, 0, 0, 1, 1};
+        return;
+    }
+    // Even lanes: this CTA's first row and slab; odd ones: its end and last slab.
+    const int k = lane & 1;
+    const int bound = part.start(a, tab, c + k);
+    const int hk = slab_containing(a, tab, NHl, bound - k);
+    int c0, c1;
+    const int n = part.slab_ctas(a, tab, hk, slab_start(a, tab, hk), slab_start(a, tab, hk + 1), &c0, &c1);
+    __syncwarp();
+    if (lane == 0) {
+        out->A = bound;
+        out->hfirst = hk;
+        out->n_first = n;
+    } else if (lane == 1) {
+        out->Bc = bound;
+        out->hlast = hk;
+        out->n_last = n;
+    }
+    __syncwarp();
 }
 
 // Slabs with no rows belong to no CTA: their outputs are zero.
@@ -508,10 +529,12 @@ __device__ __noinline__ void write_empty_slabs_tc(const DecodeArgs& a, unsigned 
     const SeqTable t = seq_table_at(table, a);
 #pragma unroll 1
     for (int h = 0; h < a.B * a.Hkv; ++h)
-        if (slab_start(a, t, h) == slab_start(a, t, h + 1))
+        if (slab_start(a, t, h) == slab_start(a, t, h + 1)) {
+            if (lane == 0) *reinterpret_cast<int2*>(a.slab_parts + 2 * h) = make_int2(0, 0);
 #pragma unroll 1
             for (int j = 0; j < a.NC; ++j)
                 write_out<G>(a, h / a.Hkv, h % a.Hkv, j, make_float4(0.f, 0.f, 0.f, 0.f), 0.f, lane);
+        }
 }
 
 template <int G>
@@ -560,7 +583,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __syncthreads();
     finish_slab_cache(a, tab, kTcThreads);
     __syncthreads();
-    pdl_launch_dependents();
 
     if (warp == 0) tc_share(a, table, c, reinterpret_cast<TcShare*>(sm + kOffInfo));
     __syncthreads();
@@ -569,7 +591,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         write_empty_slabs_tc<G>(a, table, lane);
     }
     const int A = uniform(share->A), Bc = uniform(share->Bc);
-    if (A >= Bc) return;  // uniform: this CTA has no rows (no TMEM taken yet)
+    if (A >= Bc) {  // uniform: this CTA has no rows (no TMEM taken yet)
+        pdl_wait();
+        return;
+    }
     const int hfirst = uniform(share->hfirst), hend = uniform(share->hlast) + 1;
     int32_t* slot = reinterpret_cast<int32_t*>(sm + kOffSlots) + 6 * warp;
     const int NC = a.NC;
@@ -595,7 +620,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             while ((wk.more() || wv.more()) && !uniform(flags[kFlagAbort])) {
                 bool moved = false;
                 if (wk.more() && (tk < kKStages || test_phase_warp(&k_empty[tk % kKStages], ((tk / kKStages) - 1) & 1))) {
-                    if (tk == PRE && !waited) {
+                    if (tk == kTcPre && !waited) {
                         pdl_wait();  // later copies after the previous kernel, as in the other kernels
                         waited = true;
                     }
@@ -654,14 +679,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // allocates TMEM: the first score product waits for both.
             const int st = tid - 64;
             pdl_wait();  // q and the outputs belong to the previous kernel's epoch
-            const int h1 = uniform(later_segment_slab(a, table, hfirst, hend, A, Bc, 1));
+            pdl_launch_dependents();
             load_q_tc<G>(a, hfirst, sQ, st);
-            if (h1 < hend) load_q_tc<G>(a, h1, sQ + kTcQBytes, st);
             fence_proxy_async_smem();
             named_sync(kBarSoft, kTcSoft);
-            if (st == 0) {
-                mbar_arrive(smem_u32(&q_full[0]));
-                if (h1 < hend) mbar_arrive(smem_u32(&q_full[1]));
+            if (st == 0) mbar_arrive(smem_u32(&q_full[0]));
+            const int h1 = hfirst + 1 < hend ? uniform(later_segment_slab(a, table, hfirst, hend, A, Bc, 1)) : hend;
+            if (h1 < hend) {
+                load_q_tc<G>(a, h1, sQ + kTcQBytes, st);
+                fence_proxy_async_smem();
+                named_sync(kBarSoft, kTcSoft);
+                if (st == 0) mbar_arrive(smem_u32(&q_full[1]));
             }
         }
         if (warp == 1) {
@@ -981,6 +1009,23 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             named_sync(kBarSoft, kTcSoft);
             if (leader && h2 < hend) mbar_arrive(smem_u32(&q_full[seg_idx & 1]));
+            const int64_t slot_row = (int64_t)c + h;
+            if (st < NC) {
+                // Column st: how the groups' states combine, once for all 128 dimensions.
+                const float m0 = has0 ? g_max[st] : -INFINITY, m1 = has1 ? g_max[kTcMaxCols + st] : -INFINITY;
+                const float M = fmaxf(m0, m1);
+                const float f0 = has0 ? ex2(m0 - M) : 0.f, f1 = has1 ? ex2(m1 - M) : 0.f;
+                const float L = (has0 ? f0 * g_sum[st] : 0.f) + (has1 ? f1 * g_sum[kTcMaxCols + st] : 0.f);
+                g_alpha[st] = f0;
+                g_alpha[kTcMaxCols + st] = f1;
+                g_sum[st] = L;  // (only this thread read it)
+                if (!whole) __stcg(reinterpret_cast<float2*>(a.work_ml + (slot_row * NC + st) * 2), make_float2(M, L));
+            }
+            if (leader && w.rows_from_start) {
+                // For the combine: the CTAs that hold a part of the slab (none to combine for one).
+                const int n = whole ? 1 : h == hfirst ? share->n_first : share->n_last;
+                *reinterpret_cast<int2*>(a.slab_parts + 2 * h) = make_int2(c, n);
+            }
             if (gleader) {
                 bool ok = seg_ok;
                 if (ok && last_mine >= 0) ok = wait_phase(&o_done[gi], (last_mine >> 1) & 1);
@@ -998,7 +1043,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // Merge of the groups: group gi writes the columns 32 gi .. 32 gi + 31 of every dimension.
             const int oc0 = 32 * gi;
             const int bq = h / a.Hkv, g = h - bq * a.Hkv;
-            const int64_t slot = (int64_t)c + h;
             if (merge_ok && oc0 < NCpad) {
                 // O of each group = its product with P_hi + its product with P_lo, 16
                 // columns at a time (whole 32-column blocks spilled registers to local
@@ -1017,18 +1061,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     // hold kTcMaxCols columns), so that every shared-memory load of the
                     // chunk is independent of the stores: a load-use chain per column
                     // cost ~250 cycles a column under the kernel's shared-memory traffic.
-                    float ov[16], Mv[16], Lv[16];
+                    float ov[16];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        const int cc = c16 + i;
-                        const float m0 = has0 ? g_max[cc] : -INFINITY, m1 = has1 ? g_max[kTcMaxCols + cc] : -INFINITY;
-                        const float M = fmaxf(m0, m1);
-                        const float f0 = has0 ? ex2(m0 - M) : 0.f, f1 = has1 ? ex2(m1 - M) : 0.f;
+                        const float f0 = g_alpha[c16 + i], f1 = g_alpha[kTcMaxCols + c16 + i];
                         const float v0 = __uint_as_float(r0[i]) + __uint_as_float(w0[i]);
                         const float v1 = __uint_as_float(r1[i]) + __uint_as_float(w1[i]);
                         ov[i] = (has0 ? f0 * v0 : 0.f) + (has1 ? f1 * v1 : 0.f);
-                        Mv[i] = M;
-                        Lv[i] = (has0 ? f0 * g_sum[cc] : 0.f) + (has1 ? f1 * g_sum[kTcMaxCols + cc] : 0.f);
                     }
                     // Stores that skip L1 (st.global.cg): the L1 path is busy with the
                     // tiles' shared-memory traffic, and plain stores made a segment's
@@ -1039,11 +1078,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         const int cc = c16 + i;
                         if (cc < NC) {
                             if (whole) {
-                                __stcg(a.out + out_row<G>(a, bq, g, cc) * kHeadDim + dim, Lv[i] > 0.f ? ov[i] / Lv[i] : 0.f);
+                                const float L = g_sum[cc];
+                                __stcg(a.out + out_row<G>(a, bq, g, cc) * kHeadDim + dim, L > 0.f ? ov[i] / L : 0.f);
                             } else {
-                                __stcg(a.work_o + (slot * NC + cc) * kHeadDim + dim, ov[i]);
-                                if (dim == 0)
-                                    __stcg(reinterpret_cast<float2*>(a.work_ml + (slot * NC + cc) * 2), make_float2(Mv[i], Lv[i]));
+                                __stcg(a.work_o + (slot_row * NC + cc) * kHeadDim + dim, ov[i]);
                             }
                         }
                     }
@@ -1051,114 +1089,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             // g_max / g_sum are rewritten at the next segment's end, after these reads.
             named_sync(kBarSoft, kTcSoft);
-            if (merge_ok && !whole && leader) {
-                // This CTA's partial of slab h is written (the barrier above orders the
-                // other threads' stores before this thread's fence): count it in.
-                __threadfence();
-                atomicAdd(a.slab_count + (int64_t)h * kMaxCols * 2, 1);
-            }
-        }
-
-        // ---- the CTA's share of the merges of its slabs that span several CTAs
-        // (its first and its last segment; the slabs in between were whole).
-        for (int e = 0; e < 2; ++e) {
-            const int h = e == 0 ? hfirst : hend - 1;
-            if (e == 1 && h == hfirst) break;
-            const int c0 = uniform(e == 0 ? share->c0_first : share->c0_last);
-            const int nct = uniform(e == 0 ? share->n_first : share->n_last), c1 = c0 + nct - 1;
-            if (nct <= 1) continue;  // uniform: written at its segment's end
-            int32_t* ctr = a.slab_count + (int64_t)h * kMaxCols * 2;
-            if (leader) {
-                // Every CTA of the slab counts in once its partial is written; the CTAs
-                // are all resident (cooperative launch), so the count completes.
-                bool ok = !flags[kFlagAbort];
-                if (ok) {
-                    ok = false;
-                    const unsigned long long t0 = global_ns();
-                    for (int i = 1; i < kWaitSpins; ++i) {
-                        int n;
-                        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(n) : "l"(ctr) : "memory");
-                        if (n >= nct + a.merge_extra) {
-                            ok = true;
-                            break;
-                        }
-                        if ((i & 63) == 0 && global_ns() - t0 > kWaitNs) break;
-                    }
-                    if (!ok) atomicOr(a.status, kDevMergeTimeout);
-                }
-                flags[kFlagSegOk] = ok;
-            }
-            named_sync(kBarSoft, kTcSoft);
-            if (uniform(flags[kFlagSegOk])) {
-                const int k = c - c0;  // rank of this CTA among the slab's CTAs
-                const int j0 = (int)((int64_t)k * NC / nct), j1 = (int)((int64_t)(k + 1) * NC / nct);
-                const int hb = h / a.Hkv, hg = h - hb * a.Hkv;
-                // Columns j0 .. j1-1: warp (gi, quarter) takes j0 + 4 gi + quarter, then
-                // every 8th. Per round of 32 partials, lane k loads the k-th partial's
-                // (m, l) once (the weights of the round, with a running rescale when a
-                // slab has more than 32 CTAs); then each lane covers 4 dims and keeps 16
-                // partials' o in flight, so a round costs two or three L2 round trips.
-                const int ncta = c1 - c0 + 1;
-                for (int j = j0 + 4 * gi + quarter; j < j1; j += 8) {
-                    float M = -INFINITY, L = 0.f;  // L: this lane's share of the sum
-                    float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
-                    for (int k0 = 0; k0 < ncta; k0 += 32) {
-                        const int cc = c0 + k0 + lane;
-                        const bool okp = cc <= c1;
-                        const float2 ml = okp ? __ldcg(reinterpret_cast<const float2*>(a.work_ml + (((int64_t)cc + h) * NC + j) * 2))
-                                              : make_float2(-INFINITY, 0.f);
-                        float rm = ml.x;
-#pragma unroll
-                        for (int o = 16; o >= 1; o >>= 1) rm = fmaxf(rm, __shfl_xor_sync(kFull, rm, o));
-                        const float Mn = fmaxf(M, rm);
-                        const float sc = M == -INFINITY ? 0.f : ex2(M - Mn);  // rescale of the earlier rounds
-                        const float f = ml.x == -INFINITY ? 0.f : ex2(ml.x - Mn);
-                        M = Mn;
-                        L = fmaf(ml.y, f, L * sc);
-                        O.x *= sc;
-                        O.y *= sc;
-                        O.z *= sc;
-                        O.w *= sc;
-                        const int n = min(32, ncta - k0);
-                        for (int u0 = 0; u0 < n; u0 += 16) {
-                            float4 v[16];
-                            float fk[16];
-#pragma unroll
-                            for (int u = 0; u < 16; ++u) {
-                                const int k = u0 + u;
-                                fk[u] = __shfl_sync(kFull, f, k & 31);
-                                const bool okk = __shfl_sync(kFull, okp ? 1 : 0, k & 31) != 0 && k < n;
-                                v[u] = okk ? __ldcg(reinterpret_cast<const float4*>(
-                                                        a.work_o + (((int64_t)c0 + k0 + k + h) * NC + j) * kHeadDim) +
-                                                    lane)
-                                           : make_float4(0.f, 0.f, 0.f, 0.f);
-                                if (!okk) fk[u] = 0.f;
-                            }
-#pragma unroll
-                            for (int u = 0; u < 16; ++u) {
-                                O.x = fmaf(v[u].x, fk[u], O.x);
-                                O.y = fmaf(v[u].y, fk[u], O.y);
-                                O.z = fmaf(v[u].z, fk[u], O.z);
-                                O.w = fmaf(v[u].w, fk[u], O.w);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int o = 16; o >= 1; o >>= 1) L += __shfl_xor_sync(kFull, L, o);
-                    write_out<G>(a, hb, hg, j, O, L, lane);
-                }
-            }
-            named_sync(kBarSoft, kTcSoft);
-            if (leader) {
-                // The last CTA of the slab to finish its share resets the counters for
-                // the next call (every wait on the arrival count is over by then).
-                const int done = atomicAdd(ctr + 1, 1);
-                if (done == nct - 1) {
-                    ctr[0] = 0;
-                    ctr[1] = 0;
-                    __threadfence();
-                }
-            }
         }
     }
 
@@ -1189,6 +1119,98 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols));
 }
 
+// Merge of the slabs over several CTAs: one warp a (slab, column), 4 dimensions a
+// lane. The partials' (m, l), one a lane, and their o are requested together,
+// KB at a time: one round trip to L2 for the usual slab.
+constexpr int kCombineCols = 2;
+constexpr int kCombineSlabs = 64, kCombineTable = (seq_table_bytes(kCombineSlabs, kCombineSlabs) + 15) / 16 * 16;
+static_assert(kCombineCols >= 2, "the table is built by the first warp and loaded by the others");
+__device__ __forceinline__ float4 ld_cg4(const float* p)  // (volatile: all loads of a batch stay ahead of their use)
+{
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+
+template <int G>
+__global__ void __launch_bounds__(kCombineCols * 32) combine_tc_kernel(const __grid_constant__ DecodeArgs a, int groups)
+{
+    constexpr int KB = 32;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int h = blockIdx.x / groups, j = (blockIdx.x - h * groups) * kCombineCols + warp;
+    __shared__ __align__(16) unsigned char table[kCombineTable];
+    int first = 0, n = -1;
+    if (a.B * a.Hkv <= kCombineSlabs) {
+        // Few slabs: where the slab's partials are follows from the plan, before the wait
+        // (a load after it is a round trip on the way to the output).
+        const SeqTable tab = seq_table_at(table, a);
+        if (warp == 0)
+            build_seq_table(a, tab, false);
+        else
+            load_slab_cache(a, tab, 32, (kCombineCols - 1) * 32);
+        __syncthreads();
+        finish_slab_cache(a, tab, kCombineCols * 32);
+        __syncthreads();
+        const TcPart part = tc_partition(a, tab);
+        const int p0 = slab_start(a, tab, h), p1 = slab_start(a, tab, h + 1);
+        int last;
+        n = uniform(p0 < p1 ? part.slab_ctas(a, tab, h, p0, p1, &first, &last) : 0);
+        first = uniform(first);
+    }
+    pdl_wait();
+    pdl_launch_dependents();
+    if (j >= a.NC) return;
+    if (n < 0) {
+        const int2 parts = __ldcg(reinterpret_cast<const int2*>(a.slab_parts) + h);
+        first = uniform(parts.x);
+        n = uniform(parts.y);
+    }
+    if (n <= 1) return;  // empty, or written out by its one CTA
+    const int64_t base = ((int64_t)first + h) * a.NC + j;
+    const int b = h / a.Hkv, g = h - b * a.Hkv;
+    float M = -INFINITY, L = 0.f;  // L: this lane's share of the sum
+    float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int k0 = 0; k0 < n; k0 += KB) {
+        const float* po = a.work_o + (base + (int64_t)k0 * a.NC) * kHeadDim + 4 * lane;
+        const int m = min(KB, n - k0);
+        float2 ml = make_float2(-INFINITY, 0.f);
+        if (lane < m) ml = __ldcg(reinterpret_cast<const float2*>(a.work_ml + (base + (int64_t)(k0 + lane) * a.NC) * 2));
+        float4 v[KB];
+#pragma unroll
+        for (int u = 0; u < KB; ++u) {
+            // (past the last partial: the first one again, not added below)
+            v[u] = ld_cg4(po + (u < m ? (int64_t)u * a.NC * kHeadDim : 0));
+        }
+#pragma unroll
+        for (int u = 0; u < KB; ++u) asm volatile("" : "+f"(v[u].x), "+f"(v[u].y), "+f"(v[u].z), "+f"(v[u].w));
+        float Mn = fmaxf(M, ml.x);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) Mn = fmaxf(Mn, __shfl_xor_sync(kFull, Mn, o));
+        const float sc = M == -INFINITY ? 0.f : ex2(M - Mn);  // rescale of the earlier rounds
+        const float f = ml.x == -INFINITY ? 0.f : ex2(ml.x - Mn);
+        M = Mn;
+        L = fmaf(ml.y, f, L * sc);
+        O.x *= sc;
+        O.y *= sc;
+        O.z *= sc;
+        O.w *= sc;
+#pragma unroll
+        for (int u = 0; u < KB; ++u) {
+            const float fk = __shfl_sync(kFull, f, u);
+            if (u < m) {
+                O.x = fmaf(v[u].x, fk, O.x);
+                O.y = fmaf(v[u].y, fk, O.y);
+                O.z = fmaf(v[u].z, fk, O.z);
+                O.w = fmaf(v[u].w, fk, O.w);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) L += __shfl_xor_sync(kFull, L, o);
+    write_out<G>(a, b, g, j, O, L, lane);
+}
+
 template <int G>
 cudaError_t config_tc_g(int B, DecodeConfig* cfg)
 {
@@ -1212,23 +1234,12 @@ template <int G>
 cudaError_t launch_tc_g(const DecodeArgs& a, const CacheMaps& maps, const DecodeConfig& cfg, cudaStream_t st)
 {
     if (cfg.nwarps != kTcThreads / 32 || cfg.smem_bytes < tc_smem_bytes(a.B) || a.nctas < 1 || a.nctas > cfg.nctas ||
-        a.NC < 1 || a.NC > kTcMaxCols || !a.slab_count)
+        a.NC < 1 || a.NC > kTcMaxCols || !a.slab_parts)
         return cudaErrorInvalidConfiguration;
-    // Cooperative (every CTA resident: a CTA waits for the other CTAs of its slabs)
-    // and programmatic stream serialization, as the other decode kernels.
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(a.nctas);
-    lc.blockDim = dim3(kTcThreads);
-    lc.dynamicSmemBytes = cfg.smem_bytes;
-    lc.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeCooperative;
-    attr[1].val.cooperative = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 2;
-    return cudaLaunchKernelEx(&lc, decode_tc_kernel<G>, a, maps);
+    const cudaError_t e = launch_pdl(decode_tc_kernel<G>, a.nctas, kTcThreads, cfg.smem_bytes, st, a, maps);
+    if (e != cudaSuccess) return e;
+    const int groups = (a.NC + kCombineCols - 1) / kCombineCols;
+    return launch_pdl(combine_tc_kernel<G>, a.B * a.Hkv * groups, kCombineCols * 32, 0, st, a, groups);
 }
 
 }  // namespace

@@ -92,7 +92,7 @@ struct DecodeArgs {
     float* exch_o;          // fused-merge exchange: [slots][NC][128] and [slots][NC][2], every word 0 between launches
     float* exch_ml;
     float* out;             // [B][H][128]
-    int32_t* slab_count;    // [B*Hkv][cols][2] arrivals, partials written (zero between calls)
+    int32_t* slab_parts;    // [B*Hkv][2] tcgen05 kernel: first CTA and count of the CTAs that hold a part of the slab
     int32_t* status;
     int64_t rows_cap;       // rows of Kc/Vc, for the bounds-checked build; 0 when the caller does not give it
     int B, H, Hkv, G;
@@ -177,9 +177,8 @@ cudaError_t launch_decode_mma_fused(const DecodeArgs& a, const CacheMaps& maps, 
                                     cudaStream_t st);
 cudaError_t launch_advance(int32_t* n_app, int B, int reserve, int32_t* status, cudaStream_t st);
 
-// tcgen05 multi-query kernel (dkv_decode_tc.cu): 1 to kTcMaxCols columns, one CTA
-// per SM (a cooperative launch), the merge of slabs over several CTAs fused in
-// (uses a.slab_count: entry [h][0][0..1] of each slab).
+// tcgen05 multi-query kernels (dkv_decode_tc.cu): 1 to kTcMaxCols columns, one CTA
+// per SM, then the combine of the slabs over several CTAs (uses a.slab_parts).
 cudaError_t decode_config_tc(int G, int B, DecodeConfig* cfg);
 cudaError_t launch_decode_tc(const DecodeArgs& a, const CacheMaps& maps, const DecodeConfig& cfg, cudaStream_t st);
 

@@ -7,12 +7,14 @@ to many slabs a CTA; values that are exactly 0 (which must not read as "empty").
 Outputs against the fp64 oracle within the suite's tolerance; the constant-value
 cases against their closed form within 1e-5 (64 x the fp32 rounding of one sum).
 """
+import numpy as np
 import pytest
 import torch
 
+import oracle as O
 import paper_2609_32663_gb300.dkv as dkv
 from paper_2609_32663_gb300 import inputs as I
-from parity import Case
+from parity import Case, assert_close
 
 pytestmark = pytest.mark.gpu
 
@@ -78,5 +80,25 @@ def test_back_to_back_calls_are_identical():
         got = torch.cat([t.reshape(-1) for t in outs + multi])
         first = got if first is None else first
         assert torch.equal(got, first)
+    assert dkv.dkv_plan_status(c.plan) == 0
+    c.close()
+
+
+@pytest.mark.parametrize("Hkv,B,Q,T", [(8, 8, 5, 1800), (8, 9, 5, 1800), (1, 1, 16, 152 * 64 + 1), (1, 40, 5, 1500)])
+def test_combine_on_both_sides_of_the_slab_limit(Hkv, B, Q, T):
+    """17 or more columns: the combine kernel places a slab's partials itself up to
+    64 slabs a layer and reads them from the partial kernel above; also a slab over
+    every CTA (more partials than one batch)."""
+    G = 4
+    c = Case(wl(H=G * Hkv, Hkv=Hkv, B=B, T=T, W=T, seed=Q + T))
+    gen = torch.Generator().manual_seed(T)
+    q = torch.randn((B, Q, G * Hkv, 128), generator=gen).to(torch.bfloat16)
+    out = torch.full((B, Q, G * Hkv, 128), float("nan"), device=c.dev)
+    for _ in range(2):
+        dkv.dkv_decode_multi(c.plan, 0, q.to(c.dev), Q, None, c.Kc, c.Vc, out)
+    got = out.double().cpu().numpy()
+    for i in sorted({0, Q - 1}):
+        want = O.decode(c.om, 0, B, G * Hkv, Hkv, I.bf16_bits(q[:, i].contiguous()), c.oKc, c.oVc)
+        assert_close(np.ascontiguousarray(got[:, i]), want, f"query {i}")
     assert dkv.dkv_plan_status(c.plan) == 0
     c.close()
