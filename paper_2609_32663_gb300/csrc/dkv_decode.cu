@@ -676,10 +676,11 @@ cudaError_t config_g(int B, DecodeConfig* cfg)
 {
     using C = PKFor<G>;
     const int smem = C::bytes(B);
+    // (the most any plan needs: see config_mma_g)
     cudaError_t e = cudaFuncSetAttribute(decode_partial_kernel<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem);
+                                         C::bytes(kMaxB));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(decode_partial_kernel<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = cudaFuncSetAttribute(decode_partial_kernel<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::bytes(kMaxB));
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -57,7 +57,8 @@ struct MK {
     static constexpr int kFixedBytes = kRingBytes + kBarBytes + kMetaBytes;
     static int bytes(int B, int NHl) { return kAlign + kFixedBytes + seq_table_bytes(B, NHl); }
     static_assert(NS >= 2, "a K and a V half-tile");
-    static_assert(kAlign + kFixedBytes + seq_table_bytes(kMaxB) <= 227 * 1024, "fits the opt-in shared memory of one CTA");
+    static constexpr int kMaxBytes = kAlign + kFixedBytes + seq_table_bytes(kMaxB);  // the largest layer
+    static_assert(kMaxBytes <= 227 * 1024, "fits the opt-in shared memory of one CTA");
     static_assert(kDepOff + 528 <= kWarpRing, "a warp's final state and a deposit fit in its ring");
 };
 
@@ -689,13 +690,15 @@ cudaError_t config_mma_g(int B, int NHl, DecodeConfig* cfg)
     using C = MKFor<G, NT, MULTI>;
     const int smem = C::bytes(B, NHl);
     cudaError_t e;
+    // The attribute is the kernel's, not the plan's: always the most any plan needs, so
+    // that plans of other sizes keep working beside each other.
     if constexpr (!MULTI) {
         if ((e = cudaFuncSetAttribute(decode_mma_kernel<G, NT, false, false>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, C::kMaxBytes)) != cudaSuccess)
             return e;
     }
     if ((e = cudaFuncSetAttribute(decode_mma_kernel<G, NT, true, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  smem)) != cudaSuccess)
+                                  C::kMaxBytes)) != cudaSuccess)
         return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -1215,7 +1215,7 @@ template <int G>
 cudaError_t config_tc_g(int B, DecodeConfig* cfg)
 {
     const int smem = tc_smem_bytes(B);
-    cudaError_t e = cudaFuncSetAttribute(decode_tc_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(decode_tc_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_bytes(kMaxB));
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

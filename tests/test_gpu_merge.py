@@ -102,3 +102,21 @@ def test_combine_on_both_sides_of_the_slab_limit(Hkv, B, Q, T):
         assert_close(np.ascontiguousarray(got[:, i]), want, f"query {i}")
     assert dkv.dkv_plan_status(c.plan) == 0
     c.close()
+
+
+def test_plans_of_other_sizes_side_by_side():
+    """A plan keeps working after plans of the same group size but fewer sequences
+    or KV heads were made (a kernel's shared-memory limit is the kernel's, not a
+    plan's)."""
+    big = Case(wl(H=4 * 16, Hkv=16, T=1300, B=20), reserve=2)
+    small = [Case(wl(H=4 * h, Hkv=h, T=1300, B=b), reserve=2) for h, b in ((1, 1), (8, 1), (2, 3))]
+    q = torch.zeros((20, 5, 64, 128), dtype=torch.bfloat16, device=big.dev)
+    for c in [big] + small:
+        c.decode_steps(1, append=True)
+    for Q in (1, 2, 4, 5):  # every multi-query kernel
+        qq = q[:, :Q].contiguous()
+        out = torch.empty(qq.shape, device=big.dev)
+        dkv.dkv_decode_multi(big.plan, 0, qq, Q, None, big.Kc, big.Vc, out)
+    big.decode_steps(1, append=False)
+    for c in [big] + small:
+        c.close()
