@@ -4,6 +4,7 @@
 // dkv_decode_mma.cu, dkv_decode.cu and dkv_topk.cu.
 #include "dkv.h"
 #include "dkv_internal.cuh"
+#include "dkv_pool.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -11,7 +12,10 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <new>
+#include <tuple>
 #include <vector>
 
 struct dkv_plan {
@@ -24,8 +28,8 @@ struct dkv_plan {
     int64_t total_rows = 0;   // rows of the packed (or dense) cache
     int64_t kept_rows = 0;
     int device = 0;
-    void* d_arena = nullptr;    // one allocation: the map's metadata and counters (the workspace too, dense plans)
-    void* d_arena2 = nullptr;   // map plans: the index list and the workspace, sized after the map's one sync
+    dkv::PlanMemory arena{};    // one allocation: the map's metadata and counters (the workspace too, dense plans)
+    dkv::PlanMemory arena2{};   // map plans: the index list and the workspace, sized after the map's one sync
     int32_t* d_len = nullptr;   // [NH]
     int64_t* d_off = nullptr;   // [NH+1]
     int64_t* d_ioff = nullptr;  // [NH+1]
@@ -88,18 +92,15 @@ dkv_status cuda_fail(cudaError_t e, const char* where)
     return fail(DKV_ERR_CUDA, "%s: %s", where, cudaGetErrorString(e));
 }
 
-template <class T>
-dkv_status dalloc(T** p, size_t count, const char* what)
+dkv_status dalloc(dkv::PlanMemory* m, size_t bytes, const char* what)
 {
-    *p = nullptr;
-    if (count == 0) count = 1;
+    *m = dkv::PlanMemory{};
     if (fault("alloc")) return fail(DKV_ERR_OOM, "%s: injected allocation failure", what);
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), count * sizeof(T));
+    const cudaError_t e = dkv::plan_alloc(m, std::max<size_t>(bytes, 1));
     if (e != cudaSuccess) {
         cudaGetLastError();
-        *p = nullptr;
-        return fail(e == cudaErrorMemoryAllocation ? DKV_ERR_OOM : DKV_ERR_CUDA, "%s: cudaMalloc(%zu B): %s",
-                    what, count * sizeof(T), cudaGetErrorString(e));
+        return fail(e == cudaErrorMemoryAllocation ? DKV_ERR_OOM : DKV_ERR_CUDA, "%s: allocation of %zu B: %s", what, bytes,
+                    cudaGetErrorString(e));
     }
     return DKV_OK;
 }
@@ -113,11 +114,12 @@ dkv_status launched(cudaError_t e, const char* where)
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// The device must have finished the plan's work (a plan that failed half-way: its stream).
 void release(dkv_plan* p)
 {
     if (!p) return;
-    cudaFree(p->d_arena);
-    cudaFree(p->d_arena2);
+    dkv::plan_free(p->arena);
+    dkv::plan_free(p->arena2);
     delete p;
 }
 
@@ -139,6 +141,20 @@ dkv_status check_shape(const dkv_shape* s, int32_t B)
     return DKV_OK;
 }
 
+// Every byte is 0 or 1 (eight at a time: a pattern has 10^5 entries).
+bool all_binary(const uint8_t* M, size_t n)
+{
+    uint64_t bad = 0;
+    size_t i = 0;
+    for (; i + 8 <= n; i += 8) {
+        uint64_t w;
+        std::memcpy(&w, M + i, 8);
+        bad |= w & 0xfefefefefefefefeull;
+    }
+    for (; i < n; ++i) bad |= M[i] & 0xfeu;
+    return bad == 0;
+}
+
 // Byte offsets of the plan's device arrays inside its one allocation, each on a
 // 256-byte boundary.
 struct ArenaLayout {
@@ -158,20 +174,52 @@ T* at(void* base, size_t off)
     return reinterpret_cast<T*>(static_cast<unsigned char*>(base) + off);
 }
 
-// Launch configurations of every decode kernel a plan may run (host queries,
-// no device work), and the split-K workspace that serves all of them: slots for
-// the largest grid plus the slabs of a layer, warp records for the largest grid
-// x warps, kMaxCols columns.
+// Launch configurations of every decode kernel a plan may run, looked up once for
+// each (context, G, B, H_kv): some twenty runtime calls set kernel attributes and
+// query occupancy (30 us).
+struct KernelConfigs {
+    dkv::DecodeConfig f32, mma, multi1, multi, tc;
+};
+
+cudaError_t kernel_configs(int G, int B, int Hkv, KernelConfigs* out)
+{
+    static std::mutex mu;
+    static std::map<std::tuple<unsigned long long, int, int, int>, KernelConfigs> known;
+    unsigned long long id = 0;
+    cudaError_t e = dkv::current_context_id(&id);
+    if (e != cudaSuccess) return e;
+    const auto key = std::make_tuple(id, G, B, Hkv);
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find(key);
+    if (it != known.end()) {
+        *out = it->second;
+        return cudaSuccess;
+    }
+    KernelConfigs k{};
+    if ((e = dkv::decode_config(G, B, &k.f32)) != cudaSuccess ||
+        (e = dkv::decode_config_mma(G, B, Hkv, 0, &k.mma)) != cudaSuccess ||
+        (e = dkv::decode_config_mma(G, B, Hkv, 1, &k.multi1)) != cudaSuccess ||
+        (e = dkv::decode_config_mma(G, B, Hkv, 2, &k.multi)) != cudaSuccess ||
+        (e = dkv::decode_config_tc(G, B, &k.tc)) != cudaSuccess)
+        return e;
+    known.emplace(key, k);
+    *out = k;
+    return cudaSuccess;
+}
+
+// A plan's kernels (host queries, no device work), and the split-K workspace that
+// serves all of them: slots for the largest grid plus the slabs of a layer, warp
+// records for the largest grid x warps, kMaxCols columns.
 dkv_status plan_configs(dkv_plan* p)
 {
-    cudaGetDevice(&p->device);
-    cudaError_t e;
-    if ((e = dkv::decode_config(p->G, p->B, &p->cfg_f32)) != cudaSuccess) return cuda_fail(e, "decode_config");
-    if ((e = dkv::decode_config_mma(p->G, p->B, p->s.H_kv, 0, &p->cfg_mma)) != cudaSuccess ||
-        (e = dkv::decode_config_mma(p->G, p->B, p->s.H_kv, 1, &p->cfg_multi1)) != cudaSuccess ||
-        (e = dkv::decode_config_mma(p->G, p->B, p->s.H_kv, 2, &p->cfg_multi)) != cudaSuccess)
-        return cuda_fail(e, "decode_config (tensor cores)");
-    if ((e = dkv::decode_config_tc(p->G, p->B, &p->cfg_tc)) != cudaSuccess) return cuda_fail(e, "decode_config (tcgen05)");
+    KernelConfigs k;
+    const cudaError_t e = kernel_configs(p->G, p->B, p->s.H_kv, &k);
+    if (e != cudaSuccess) return cuda_fail(e, "launch configurations of the decode kernels");
+    p->cfg_f32 = k.f32;
+    p->cfg_mma = k.mma;
+    p->cfg_multi1 = k.multi1;
+    p->cfg_multi = k.multi;
+    p->cfg_tc = k.tc;
     // Warp records: the mma.sync and fp32 kernels (up to kMaxCols columns); CTA
     // partials: every kernel, up to kTcMaxCols columns (the tcgen05 kernel).
     int64_t ctas = p->cfg_tc.nctas, warp_records = 0;
@@ -203,7 +251,7 @@ ZeroBlock take_zeroed(ArenaLayout& lay, const dkv_plan* p, size_t extra)
 
 void place_zeroed(dkv_plan* p, const ZeroBlock& z)
 {
-    p->d_status = at<int32_t>(p->d_arena, z.off);
+    p->d_status = at<int32_t>(p->arena.ptr, z.off);
     p->d_slab_parts = p->d_status + 2;  // 8-byte aligned
 }
 
@@ -257,8 +305,9 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     if (st != DKV_OK) return st;
     if (reserve_rows < 0) return fail(DKV_ERR_INVALID_ARG, "reserve_rows=%d < 0", reserve_rows);
     const size_t nM = (size_t)s->L * s->H * s->D;
-    for (size_t i = 0; i < nM; ++i)
-        if (M_host[i] > 1) return fail(DKV_ERR_INVALID_ARG, "M[%zu]=%u is not 0/1", i, M_host[i]);
+    if (!all_binary(M_host, nM))
+        for (size_t i = 0; i < nM; ++i)
+            if (M_host[i] > 1) return fail(DKV_ERR_INVALID_ARG, "M[%zu]=%u is not 0/1", i, M_host[i]);
     int32_t Tmax = 0;
     for (int b = 0; b < B; ++b) {
         const int32_t T = ctx_len_host[b];
@@ -292,7 +341,9 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     p->reserve = reserve_rows;
     p->inplace_stride = inplace_stride;
     p->T_stride = inplace_stride;
+    cudaGetDevice(&p->device);
     auto bail = [&](dkv_status e) {
+        cudaStreamSynchronize(stream);  // kernels and copies into the plan's memory
         release(p);
         return e;
     };
@@ -301,37 +352,35 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     const size_t o_len = lay.take<int32_t>((size_t)NH), o_off = lay.take<int64_t>((size_t)NH + 1),
                  o_ioff = lay.take<int64_t>((size_t)NH + 1), o_nruns = lay.take<int32_t>((size_t)NH),
                  o_runs = lay.take<int2>((size_t)NH * (s->D + 2)), o_tail = lay.take<int64_t>((size_t)3 + s->L),
-                 o_M = lay.take<uint8_t>(nM), o_Tc = lay.take<int32_t>((size_t)B),
                  o_order = inplace_stride > 0 ? lay.take<int32_t>((size_t)NH + 1) : 0;
+    // What the host gives: the counters' zeros, the pattern and the lengths, one copy.
     const ZeroBlock zb = take_zeroed(lay, p, 1);  // + the runs kernel's CTA counter
-    if ((st = dalloc(reinterpret_cast<unsigned char**>(&p->d_arena), lay.bytes, "plan metadata")) != DKV_OK)
+    const size_t o_M = lay.take<uint8_t>(nM), o_Tc = lay.take<int32_t>((size_t)B);
+    if ((st = dalloc(&p->arena, lay.bytes, "plan metadata")) != DKV_OK)
         return bail(st);
-    p->d_len = at<int32_t>(p->d_arena, o_len);
-    p->d_off = at<int64_t>(p->d_arena, o_off);
-    p->d_ioff = at<int64_t>(p->d_arena, o_ioff);
-    p->d_order = inplace_stride > 0 ? at<int32_t>(p->d_arena, o_order) : nullptr;
+    p->d_len = at<int32_t>(p->arena.ptr, o_len);
+    p->d_off = at<int64_t>(p->arena.ptr, o_off);
+    p->d_ioff = at<int64_t>(p->arena.ptr, o_ioff);
+    p->d_order = inplace_stride > 0 ? at<int32_t>(p->arena.ptr, o_order) : nullptr;
     place_zeroed(p, zb);
 
     cudaError_t e;
-    if ((e = cudaMemsetAsync(p->d_status, 0, zb.count * sizeof(int32_t), stream)) != cudaSuccess)
-        return bail(cuda_fail(e, "clear counters"));
-    if (nM && (e = cudaMemcpyAsync(at<uint8_t>(p->d_arena, o_M), M_host, nM, cudaMemcpyHostToDevice, stream)) !=
-                  cudaSuccess)
-        return bail(cuda_fail(e, "copy pattern"));
-    if ((e = cudaMemcpyAsync(at<int32_t>(p->d_arena, o_Tc), ctx_len_host, (size_t)B * 4, cudaMemcpyHostToDevice,
-                             stream)) != cudaSuccess)
-        return bail(cuda_fail(e, "copy ctx_len"));
+    std::vector<uint8_t> given(lay.bytes - zb.off);
+    if (nM) std::memcpy(given.data() + (o_M - zb.off), M_host, nM);
+    std::memcpy(given.data() + (o_Tc - zb.off), ctx_len_host, (size_t)B * 4);
+    if ((e = cudaMemcpyAsync(p->d_status, given.data(), given.size(), cudaMemcpyHostToDevice, stream)) != cudaSuccess)
+        return bail(cuda_fail(e, "copy pattern and lengths"));
 
     dkv::MapArgs ma{};
-    ma.M = at<uint8_t>(p->d_arena, o_M);
-    ma.Tc = at<int32_t>(p->d_arena, o_Tc);
-    ma.runs = at<int2>(p->d_arena, o_runs);
-    ma.nruns = at<int32_t>(p->d_arena, o_nruns);
+    ma.M = at<uint8_t>(p->arena.ptr, o_M);
+    ma.Tc = at<int32_t>(p->arena.ptr, o_Tc);
+    ma.runs = at<int2>(p->arena.ptr, o_runs);
+    ma.nruns = at<int32_t>(p->arena.ptr, o_nruns);
     ma.len = p->d_len;
     ma.off = p->d_off;
     ma.ioff = p->d_ioff;
     ma.idx = nullptr;
-    ma.tail = at<int64_t>(p->d_arena, o_tail);
+    ma.tail = at<int64_t>(p->arena.ptr, o_tail);
     ma.done = reinterpret_cast<unsigned*>(p->d_status + zb.count - 1);
     ma.order = p->d_order;
     ma.L = s->L;
@@ -360,12 +409,12 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     ArenaLayout lay2;
     const size_t o_idx = lay2.take<int32_t>((size_t)p->kept_rows), o_work = lay2.take<float>((size_t)p->work.total),
                  o_exch = lay2.take<float>((size_t)exch_floats(p));
-    if ((st = dalloc(reinterpret_cast<unsigned char**>(&p->d_arena2), lay2.bytes, "index list and workspace")) !=
+    if ((st = dalloc(&p->arena2, lay2.bytes, "index list and workspace")) !=
         DKV_OK)
         return bail(st);
-    p->d_idx = at<int32_t>(p->d_arena2, o_idx);
-    p->d_work = at<float>(p->d_arena2, o_work);
-    p->d_exch = at<float>(p->d_arena2, o_exch);
+    p->d_idx = at<int32_t>(p->arena2.ptr, o_idx);
+    p->d_work = at<float>(p->arena2.ptr, o_work);
+    p->d_exch = at<float>(p->arena2.ptr, o_exch);
     if ((e = cudaMemsetAsync(p->d_exch, 0, (size_t)exch_floats(p) * sizeof(float), stream)) != cudaSuccess)
         return bail(cuda_fail(e, "clear exchange"));
     ma.idx = p->d_idx;
@@ -415,8 +464,10 @@ dkv_status dkv_plan_dense(const int32_t* ctx_len_host, int32_t B, const dkv_shap
     p->G = s->H / s->H_kv;
     p->dense = 1;
     p->T_stride = T_stride;
+    cudaGetDevice(&p->device);
     p->reserve = (int)(T_stride - Tmax);
     auto bail = [&](dkv_status e) {
+        cudaStreamSynchronize(stream);
         release(p);
         return e;
     };
@@ -445,13 +496,13 @@ dkv_status dkv_plan_dense(const int32_t* ctx_len_host, int32_t B, const dkv_shap
                  o_ioff = lay.take<int64_t>((size_t)NH + 1);
     const ZeroBlock zb = take_zeroed(lay, p, 0);
     const size_t o_work = lay.take<float>((size_t)p->work.total), o_exch = lay.take<float>((size_t)exch_floats(p));
-    if ((st = dalloc(reinterpret_cast<unsigned char**>(&p->d_arena), lay.bytes, "plan metadata")) != DKV_OK)
+    if ((st = dalloc(&p->arena, lay.bytes, "plan metadata")) != DKV_OK)
         return bail(st);
-    p->d_len = at<int32_t>(p->d_arena, o_len);
-    p->d_off = at<int64_t>(p->d_arena, o_off);
-    p->d_ioff = at<int64_t>(p->d_arena, o_ioff);
-    p->d_work = at<float>(p->d_arena, o_work);
-    p->d_exch = at<float>(p->d_arena, o_exch);
+    p->d_len = at<int32_t>(p->arena.ptr, o_len);
+    p->d_off = at<int64_t>(p->arena.ptr, o_off);
+    p->d_ioff = at<int64_t>(p->arena.ptr, o_ioff);
+    p->d_work = at<float>(p->arena.ptr, o_work);
+    p->d_exch = at<float>(p->arena.ptr, o_exch);
     place_zeroed(p, zb);
     cudaError_t e;
     if ((e = cudaMemsetAsync(p->d_status, 0, zb.count * sizeof(int32_t), stream)) != cudaSuccess ||
@@ -776,8 +827,13 @@ dkv_status dkv_plan_status(const dkv_plan* p, int32_t* word, int32_t clear, cuda
 void dkv_free(dkv_plan* p)
 {
     if (!p) return;
+    // The plan's own device, whichever is current: its memory may serve the next plan at once.
+    int dev = p->device;
+    const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != p->device;
+    if (other) cudaSetDevice(p->device);
     cudaDeviceSynchronize();
     release(p);
+    if (other) cudaSetDevice(dev);
 }
 
 }  // extern "C"

@@ -15,8 +15,7 @@
 // streams, or different host threads) race on the array.
 #include "dkv.h"
 #include "dkv_internal.cuh"
-
-#include <cuda.h>
+#include "dkv_pool.cuh"
 
 #include <cmath>
 #include <cstdarg>
@@ -42,49 +41,16 @@ static __device__ __align__(256) unsigned char g_decode_scratch[kScratchBytes];
 //     host-side stand-in, never the device memory);
 //   - the fp32 decode kernel's launch configuration for each (G, B), so that a
 //     call does not set kernel attributes and query occupancy every time.
-using CtxGetCurrentFn = CUresult (*)(CUcontext*);
-using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long*);
-
 std::mutex g_setup_mu;
 std::vector<std::pair<unsigned long long, void*>> g_scratch_addr;  // (context ID, device address)
 std::map<std::tuple<unsigned long long, int, int>, dkv::DecodeConfig> g_configs;  // (context ID, G, B)
-
-template <class F>
-F driver_fn(const char* name)
-{
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-        return nullptr;
-    return reinterpret_cast<F>(p);
-}
-
-// ID of the calling thread's current context; the runtime's primary context of
-// the current device is made current first if none is.
-cudaError_t current_context_id(unsigned long long* id)
-{
-    static const CtxGetCurrentFn get_current = driver_fn<CtxGetCurrentFn>("cuCtxGetCurrent");
-    static const CtxGetIdFn get_id = driver_fn<CtxGetIdFn>("cuCtxGetId");
-    if (!get_current || !get_id) return cudaErrorNotSupported;
-    CUcontext ctx = nullptr;
-    if (get_current(&ctx) != CUDA_SUCCESS) return cudaErrorDeviceUninitialized;
-    if (!ctx) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaSetDevice(dev);  // initialises the device's primary context
-        if (e != cudaSuccess) return e;
-        if (get_current(&ctx) != CUDA_SUCCESS || !ctx) return cudaErrorDeviceUninitialized;
-    }
-    return get_id(ctx, id) == CUDA_SUCCESS ? cudaSuccess : cudaErrorDeviceUninitialized;
-}
 
 // The device address of the array and the launch configuration for (G, B) in
 // the current context, looked up on the context's first call.
 cudaError_t setup_for_current_context(int G, int B, void** scratch, dkv::DecodeConfig* cfg)
 {
     unsigned long long id = 0;
-    cudaError_t e = current_context_id(&id);
+    cudaError_t e = dkv::current_context_id(&id);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lk(g_setup_mu);
     void* addr = nullptr;
