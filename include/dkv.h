@@ -364,7 +364,10 @@ void dkv_free(dkv_plan* plan);
  *                bytes, 4-byte aligned; calls that share it must be ordered.
  *                Its first 32-bit word is a status word: nonzero after a call
  *                whose grid barrier wait ran out (M is then incomplete).
- *                One cooperative launch (all its CTAs resident at once).
+ *                Up to 262,144 entries one launch of a thread-block cluster, which
+ *                may start while the previous kernel in the stream still runs and
+ *                reads P only after it has completed; more entries, one cooperative
+ *                launch (all its CTAs resident at once).
  *                Asynchronous on stream; allocates nothing.
  * Errors: DKV_ERR_INVALID_ARG (n < 0 or n >= 2^31, K outside [0, n], a NULL
  * pointer with n > 0, a small or unaligned workspace), DKV_ERR_CUDA.

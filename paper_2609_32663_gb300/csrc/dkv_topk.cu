@@ -2,7 +2,8 @@
 // largest of the n entries of P set to 1. Ties go to the lower flat index and
 // NaN ranks below every number (+0 and -0 tie).
 //
-// One cooperative launch: a radix select over an order-preserving 32-bit key of
+// Up to kClEntries entries go to the one-cluster kernel further down. More: one
+// cooperative launch, a radix select over an order-preserving 32-bit key of
 // each value, in phases separated by grid barriers. CTA c owns the contiguous
 // index range [lo_c, hi_c) (its warps equal parts of it) and reads it in
 // phases 1, 2, 3 and 5 (from L2 after the first, while P fits there).
@@ -22,6 +23,8 @@
 // are long), and a CTA adds its nonzero bins to the global histogram.
 #include "dkv.h"
 #include "dkv_internal.cuh"
+
+#include <cooperative_groups.h>
 
 #include <cstdint>
 #include <mutex>
@@ -260,6 +263,252 @@ __global__ void __launch_bounds__(kTkThreads) topk_kernel(const float* __restric
     });
 }
 
+// ------------------------------------------------------------ one cluster
+// The same select for patterns that one cluster of 8 CTAs holds in registers (KPT
+// keys a thread). What bounds the kernel above on those is the latency of its
+// phases: a memset launch, a cooperative launch, and four barriers through L2 with P
+// and the histograms read through L2 between them. Here P is read once, a phase ends
+// in the hardware's cluster barrier, and a digit's histogram of all keys lives in the
+// CTAs' shared memory: bin b in CTA b % 8, so that the few bins of a narrow range of
+// values spread over the CTAs. (Every CTA reading all eight histograms and adding them
+// up, without remote atomics, was slower: 16.2 us at 131,072 entries.)
+//
+// A CTA counts in kCopies copies of its histogram, lane by lane: the first digit is
+// the sign, the exponent and two bits, a dozen bins for probabilities, and without
+// copies a warp's lanes would queue for them. Copy c is rotated by 8 c words, so that
+// a bin's copies lie in different banks.
+//
+// A unit of 128 entries is a warp's step, 4 consecutive ones a lane: 16-byte loads and
+// 4-byte stores where P and M are aligned for them. The launch overlaps its start with
+// the end of the previous kernel.
+//
+// us a call, grid-wide kernel and this one, probabilities: 1,536 entries 18.9 -> 7.6,
+// 65,536 22.6 -> 8.8, 131,072 22.6 -> 11.6, 262,144 23.9 -> 18.6; any bit pattern as
+// probabilities within 6 %. (Clusters of 16 CTAs x 512 threads: 11.6 at 131,072 but 14.9
+// for uniform bit patterns, whose 2,048 bins are all remote additions; 8 x 512 12.8, 4 x
+// 1,024 17.3.)
+constexpr int kClCtas = 8, kClThreads = 1024, kClWarps = kClThreads / 32;
+constexpr int kClBins = 2048, kCopies = 4, kClUnit = 128;
+constexpr int kClSmem = kCopies * kClBins * 4;
+constexpr int kClOwn = kClBins / kClCtas;
+
+template <int KPT>
+__global__ void __launch_bounds__(kClThreads, 1) topk_cluster_kernel(const float* __restrict__ P, int n, uint32_t K,
+                                                                     uint8_t* __restrict__ M, uint32_t* ws)
+{
+    namespace cg = cooperative_groups;
+    constexpr int U = KPT / 4;                        // units a warp
+    extern __shared__ __align__(16) uint32_t hist[];  // [kCopies][kClBins]
+    __shared__ uint32_t tot[3][kClOwn];               // of each digit: this CTA's bins of the whole histogram
+    __shared__ uint32_t warp_sum[kClWarps], wties[kClWarps], cta_ties[kClCtas];
+    __shared__ uint32_t sel_bin, sel_rank;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int rank = (int)cluster.block_rank();
+    // The units of CTA `rank`, and of them those of this warp: at most U.
+    const int units = (n + kClUnit - 1) / kClUnit;
+    const int u0 = units * rank / kClCtas, u1 = units * (rank + 1) / kClCtas;
+    const int wlo = kClUnit * (u0 + (u1 - u0) * warp / kClWarps) + 4 * lane;  // the lane's first entry
+    const int whi = min(n, kClUnit * (u0 + (u1 - u0) * (warp + 1) / kClWarps));
+    const bool vec_p = (reinterpret_cast<uintptr_t>(P) & 15u) == 0, vec_m = (reinterpret_cast<uintptr_t>(M) & 3u) == 0;
+
+    for (int i = t; i < kClBins * kCopies / 4; i += kClThreads) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = t; i < 3 * kClOwn; i += kClThreads) (&tot[0][0])[i] = 0u;
+    cluster.barrier_arrive();
+    // Overlaps its start with the previous kernel's end; that kernel's results are read from here on.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (rank == 0 && t == 0) ws[kWsStatus] = 0u;
+    float4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int i = wlo + kClUnit * u;
+        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (vec_p && i + 3 < whi) {
+            v[u] = __ldg(reinterpret_cast<const float4*>(P + i));
+        } else {
+            if (i < whi) v[u].x = __ldg(P + i);
+            if (i + 1 < whi) v[u].y = __ldg(P + i + 1);
+            if (i + 2 < whi) v[u].z = __ldg(P + i + 2);
+            if (i + 3 < whi) v[u].w = __ldg(P + i + 3);
+        }
+    }
+    uint32_t key[KPT];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        key[4 * u] = order_key(v[u].x);
+        key[4 * u + 1] = order_key(v[u].y);
+        key[4 * u + 2] = order_key(v[u].z);
+        key[4 * u + 3] = order_key(v[u].w);
+    }
+    const auto valid = [&](int i) { return wlo + kClUnit * (i >> 2) + (i & 3) < whi; };
+    cluster.barrier_wait();  // every CTA's bins are zero
+
+    // Digit by digit from the top: bits 31-21, 20-10, 9-0.
+    uint32_t prefix = 0, k = K;  // the bits of the K-th key known so far, and its rank among the keys that have them
+    const int copy = lane & (kCopies - 1);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        constexpr int kShift[3] = {21, 10, 0};
+        const int bits = d < 2 ? 11 : 10, shift = kShift[d], nbins = 1 << bits;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+            if (valid(i) && (d == 0 || (key[i] >> (shift + bits)) == prefix)) {
+                const uint32_t bin = (key[i] >> shift) & (uint32_t)(nbins - 1);
+                atomicAdd(hist + copy * kClBins + ((bin + 8 * copy) & (kClBins - 1)), 1u);
+            }
+        __syncthreads();
+#pragma unroll
+        for (int b = t; b < nbins; b += kClThreads) {
+            uint32_t c = 0;
+#pragma unroll
+            for (int r = 0; r < kCopies; ++r) {
+                uint32_t* h = hist + r * kClBins + ((b + 8 * r) & (kClBins - 1));
+                c += *h;
+                *h = 0u;  // for the next digit
+            }
+            if (c) atomicAdd(cluster.map_shared_rank(&tot[d][b / kClCtas], b % kClCtas), c);
+        }
+        cluster.sync();
+        // The bin that holds rank k, counted from the largest down, and the rank inside
+        // it. Thread t has the q bins nbins - 1 - q t downwards.
+        const int q = nbins / kClThreads;
+        uint32_t c[kClBins / kClThreads], sum = 0;
+#pragma unroll
+        for (int i = 0; i < q; ++i) {
+            const int b = nbins - 1 - q * t - i;
+            c[i] = *cluster.map_shared_rank(&tot[d][b / kClCtas], b % kClCtas);
+            sum += c[i];
+        }
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += x;
+        }
+        if (lane == 31) warp_sum[warp] = incl;
+        __syncthreads();
+        const uint32_t excl = __reduce_add_sync(kFull, lane < warp ? warp_sum[lane & (kClWarps - 1)] : 0u) + incl - sum;
+        if (excl < k && excl + sum >= k) {  // exactly one thread
+            uint32_t above = excl;
+            bool found = false;
+#pragma unroll
+            for (int i = 0; i < q; ++i) {
+                if (!found && above + c[i] >= k) {
+                    sel_bin = (uint32_t)(nbins - 1 - q * t - i);
+                    sel_rank = k - above;
+                    found = true;
+                }
+                above += c[i];
+            }
+        }
+        __syncthreads();
+        prefix = (prefix << bits) | sel_bin;
+        k = sel_rank;
+    }
+
+    // The threshold key is prefix; the first k keys equal to it are taken, in index order.
+    uint32_t ties = 0;  // bit i: key i of this thread is one
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) ties |= valid(i) && key[i] == prefix ? 1u << i : 0u;
+    const uint32_t of_warp = __reduce_add_sync(kFull, (uint32_t)__popc(ties));
+    if (lane == 0) wties[warp] = of_warp;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t all = __reduce_add_sync(kFull, lane < kClWarps ? wties[lane] : 0u);
+        if (lane < kClCtas) *cluster.map_shared_rank(&cta_ties[rank], lane) = all;
+    }
+    cluster.sync();  // the last access to another CTA's shared memory is before it
+    uint32_t carry =
+        __reduce_add_sync(kFull, (lane < warp ? wties[lane & (kClWarps - 1)] : 0u) + (lane < rank ? cta_ties[lane & (kClCtas - 1)] : 0u));
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const uint32_t here = (ties >> (4 * u)) & 15u;
+        uint32_t take = 0;  // the lane's ties of this unit that are taken
+        if (__any_sync(kFull, here != 0)) {
+            uint32_t incl = __popc(here);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t x = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += x;
+            }
+            uint32_t before = carry + incl - __popc(here);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if ((here >> j) & 1u) take |= before++ < k ? 1u << j : 0u;
+            carry += __shfl_sync(kFull, incl, 31);
+        }
+        uchar4 m;
+        m.x = key[4 * u] > prefix || (take & 1u);
+        m.y = key[4 * u + 1] > prefix || (take & 2u);
+        m.z = key[4 * u + 2] > prefix || (take & 4u);
+        m.w = key[4 * u + 3] > prefix || (take & 8u);
+        const int i = wlo + kClUnit * u;
+        if (vec_m && i + 3 < whi) {
+            *reinterpret_cast<uchar4*>(M + i) = m;
+        } else {
+            if (i < whi) M[i] = m.x;
+            if (i + 1 < whi) M[i + 1] = m.y;
+            if (i + 2 < whi) M[i + 2] = m.z;
+            if (i + 3 < whi) M[i + 3] = m.w;
+        }
+    }
+}
+
+// The most entries: 32 keys a thread. Beyond, 16 CTAs would be needed, which is a cluster
+// size that a device need not have, for 28.7 -> 25.7 us at 393,216.
+constexpr int kClMaxKeys = 32;
+constexpr int kClEntries = kClCtas * kClThreads * kClMaxKeys;
+
+using TopkClusterFn = void (*)(const float*, int, uint32_t, uint8_t*, uint32_t*);
+TopkClusterFn cluster_kernel(int64_t n)
+{
+    // The fewest keys a thread that hold n: every one is a step of each loop (131,072
+    // entries 11.6 us with 16, 65,536 8.8 with 8).
+    return n <= kClCtas * kClThreads * 8    ? topk_cluster_kernel<8>
+           : n <= kClCtas * kClThreads * 16 ? topk_cluster_kernel<16>
+                                            : topk_cluster_kernel<kClMaxKeys>;
+}
+
+void cluster_config(cudaLaunchConfig_t* lc, cudaLaunchAttribute* attr, cudaStream_t st)
+{
+    *lc = {};
+    lc->gridDim = dim3(kClCtas);
+    lc->blockDim = dim3(kClThreads);
+    lc->dynamicSmemBytes = kClSmem;
+    lc->stream = st;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = kClCtas;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    lc->attrs = attr;
+    lc->numAttrs = 2;
+}
+
+// The kernels' attributes, and whether the device (or this process's share of it)
+// can run a cluster of this size.
+cudaError_t setup_cluster(bool* usable)
+{
+    *usable = true;
+    for (const int64_t n : {(int64_t)1, (int64_t)kClEntries / 2, (int64_t)kClEntries}) {
+        const TopkClusterFn f = cluster_kernel(n);
+        cudaError_t e;
+        if ((e = cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, kClSmem)) != cudaSuccess)
+            return e;
+        cudaLaunchConfig_t lc;
+        cudaLaunchAttribute attr[2];
+        cluster_config(&lc, attr, nullptr);
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, (const void*)f, &lc) != cudaSuccess) {
+            cudaGetLastError();
+            clusters = 0;
+        }
+        *usable = *usable && clusters > 0;
+    }
+    return cudaSuccess;
+}
+
 }  // namespace
 
 int64_t topk_workspace_bytes() { return (int64_t)kWsWords * 4; }
@@ -271,14 +520,15 @@ cudaError_t launch_topk(const float* P, int64_t n, int64_t K, uint8_t* M, void* 
     if (n == 0) return cudaSuccess;
     if (K == 0 || K == n) return cudaMemsetAsync(M, K == n ? 1 : 0, (size_t)n, st);
     uint32_t* ws = static_cast<uint32_t*>(workspace);
-    if ((e = cudaMemsetAsync(ws, 0, sizeof(uint32_t) * kWsZeroed, st)) != cudaSuccess) return e;
     // Device capacity, looked up once per device (the host cost of these calls
     // would otherwise dominate small exports).
     static std::mutex mu;
     static int cached_dev = -1, cached_cap = 0;
+    static bool cached_cluster = false;
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     int64_t cap = 0;
+    bool cluster = false;
     {
         std::lock_guard<std::mutex> lock(mu);
         if (cached_dev != dev) {
@@ -290,11 +540,21 @@ cudaError_t launch_topk(const float* P, int64_t n, int64_t K, uint8_t* M, void* 
             if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, topk_kernel, kTkThreads, kTkSmem)) !=
                 cudaSuccess)
                 return e;
+            if ((e = setup_cluster(&cached_cluster)) != cudaSuccess) return e;
             cached_cap = sms * (per_sm < 1 ? 1 : per_sm);
             cached_dev = dev;
         }
         cap = cached_cap;
+        cluster = cached_cluster;
     }
+    // (The barrier's fault injection is the other kernel's.)
+    if (cluster && n <= kClEntries && !phantom_cta) {
+        cudaLaunchConfig_t lc;
+        cudaLaunchAttribute attr[2];
+        cluster_config(&lc, attr, st);
+        return cudaLaunchKernelEx(&lc, cluster_kernel(n), P, (int)n, (uint32_t)K, M, ws);
+    }
+    if ((e = cudaMemsetAsync(ws, 0, sizeof(uint32_t) * kWsZeroed, st)) != cudaSuccess) return e;
     // Every CTA must be resident at once (grid barriers): at most the device's
     // capacity, and no more CTAs than ranges of kTkMinPerCta entries.
     const int64_t want = (n + kTkMinPerCta - 1) / kTkMinPerCta;
