@@ -114,12 +114,12 @@ dkv_status launched(cudaError_t e, const char* where)
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// The device must have finished the plan's work (a plan that failed half-way: its stream).
-void release(dkv_plan* p)
+// idle: the device is known to have finished the plan's work.
+void release(dkv_plan* p, bool idle)
 {
     if (!p) return;
-    dkv::plan_free(p->arena);
-    dkv::plan_free(p->arena2);
+    dkv::plan_free(p->arena, idle);
+    dkv::plan_free(p->arena2, idle);
     delete p;
 }
 
@@ -343,8 +343,7 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     p->T_stride = inplace_stride;
     cudaGetDevice(&p->device);
     auto bail = [&](dkv_status e) {
-        cudaStreamSynchronize(stream);  // kernels and copies into the plan's memory
-        release(p);
+        release(p, cudaStreamSynchronize(stream) == cudaSuccess);  // kernels and copies into the plan's memory
         return e;
     };
 
@@ -467,8 +466,7 @@ dkv_status dkv_plan_dense(const int32_t* ctx_len_host, int32_t B, const dkv_shap
     cudaGetDevice(&p->device);
     p->reserve = (int)(T_stride - Tmax);
     auto bail = [&](dkv_status e) {
-        cudaStreamSynchronize(stream);
-        release(p);
+        release(p, cudaStreamSynchronize(stream) == cudaSuccess);
         return e;
     };
     if ((st = plan_configs(p)) != DKV_OK) return bail(st);
@@ -831,8 +829,7 @@ void dkv_free(dkv_plan* p)
     int dev = p->device;
     const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != p->device;
     if (other) cudaSetDevice(p->device);
-    cudaDeviceSynchronize();
-    release(p);
+    release(p, cudaDeviceSynchronize() == cudaSuccess);
     if (other) cudaSetDevice(dev);
 }
 

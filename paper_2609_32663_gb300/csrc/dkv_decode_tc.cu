@@ -1224,7 +1224,7 @@ cudaError_t config_tc_g(int B, DecodeConfig* cfg)
         cudaSuccess)
         return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    cfg->nctas = sms;  // one CTA per SM: co-resident (cooperative), and the TMEM allocation never waits
+    cfg->nctas = sms;  // one CTA per SM: the TMEM allocation never waits
     cfg->nwarps = kTcThreads / 32;
     cfg->smem_bytes = smem;
     return cudaSuccess;

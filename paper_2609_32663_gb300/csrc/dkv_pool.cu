@@ -4,8 +4,10 @@
 // the time of mapping and packing a 32K cache (764 us, of which 463 us are the
 // packing kernel). So the memory of a released plan is kept for the next one:
 // at most kKeepBytes a context, and all of it is given back when the context's
-// last plan is released. A plan is released only after its device has finished
-// everything, so a kept block is idle and serves any stream and thread at once.
+// last plan is released. Only a block that the device is known to have finished with is
+// kept (a wait can fail, under stream capture for one), so a kept one serves any stream
+// and thread at once; and only in its own context, which may be gone when a plan is
+// released from another.
 #include "dkv_pool.cuh"
 
 #include <cuda.h>
@@ -118,20 +120,21 @@ cudaError_t plan_alloc(PlanMemory* m, size_t bytes)
     return cudaSuccess;
 }
 
-void plan_free(const PlanMemory& m)
+void plan_free(const PlanMemory& m, bool idle)
 {
     if (!m.ptr) return;
+    unsigned long long id = 0;
+    const bool own = current_context_id(&id) == cudaSuccess && id == m.context;
     std::lock_guard<std::mutex> lock(g_mu);
     Context& c = context_of(m.context);
-    if (--c.live == 0) {
-        cudaFree(m.ptr);
-        give_back(c);
-    } else if (c.kept_bytes + m.bytes <= kKeepBytes) {
+    --c.live;
+    if (own && idle && c.live > 0 && c.kept_bytes + m.bytes <= kKeepBytes) {
         c.kept.push_back(m);
         c.kept_bytes += m.bytes;
     } else {
         cudaFree(m.ptr);
     }
+    if (own && c.live == 0) give_back(c);
 }
 
 }  // namespace dkv

@@ -17,7 +17,8 @@ struct PlanMemory {
 };
 
 cudaError_t plan_alloc(PlanMemory* m, size_t bytes);
-// No-op for none. The device must have finished all work that uses the memory.
-void plan_free(const PlanMemory& m);
+// No-op for none. idle: the device has finished all work that uses the memory (else it
+// is not kept for another plan).
+void plan_free(const PlanMemory& m, bool idle);
 
 }  // namespace dkv
