@@ -17,7 +17,6 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxB = 512;
 constexpr float kSlack = 8.f;        // lazy-rescale threshold of the online softmax (log2 units)
-constexpr int PRE = 1;               // tiles a warp fetches before waiting for the previous kernel
 
 // A value that is the same in every lane, read from lane 0. The compiler then
 // knows it is uniform over the warp: loops and branches on it are plain ones (the
@@ -202,7 +201,8 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
-// Tile cursor of one warp over its row range, with the current slab's constants.
+// Tile cursor of one warp over its row range, with the current slab's constants
+// (warp-uniform; advanced by the whole warp).
 struct Cursor {
     int h;         // slab; == hend when exhausted
     int s0, s1;    // the warp's rows of this slab, [s0, s1) (layer rows)
@@ -218,16 +218,17 @@ __device__ __forceinline__ void cursor_seek(Cursor& cu, const DecodeArgs& a, con
 {
 #pragma unroll 1
     while (cu.h < hend) {
-        cu.p0 = slab_start(a, t, cu.h);
-        const int p1 = slab_start(a, t, cu.h + 1);
+        cu.p0 = uniform(slab_start(a, t, cu.h));
+        const int p1 = uniform(slab_start(a, t, cu.h + 1));
         cu.s0 = max(wA, cu.p0);
         cu.s1 = min(wB, p1);
         if (cu.s0 < cu.s1) {
             const int b = cu.h / a.Hkv;
             const int e = t.NP[b + 1] - t.NP[b];
+            const int64_t base = t.OFF ? t.OFF[cu.h] : a.off[cu.h];
             cu.n_h = p1 - cu.p0;
-            cu.app = (a.append && e > t.NA[b]) ? 1 : 0;
-            cu.base = t.OFF ? t.OFF[cu.h] : a.off[cu.h];
+            cu.app = uniform((a.append && e > t.NA[b]) ? 1 : 0);
+            cu.base = (int64_t)(((uint64_t)(uint32_t)uniform((int)(base >> 32)) << 32) | (uint32_t)uniform((int)base));
             cu.x = cu.s0;
             return;
         }
