@@ -577,9 +577,9 @@ dkv_status dkv_vmm_trim(dkv_vmm* m, const dkv_plan* p, int32_t guard_rows, int64
     if (freed_bytes) *freed_bytes = 0;
     if (!m || !p) return fail(DKV_ERR_INVALID_ARG, "NULL buffer or plan");
     if (p->inplace_stride <= 0) return fail(DKV_ERR_INVALID_ARG, "dkv_vmm_trim needs a plan from dkv_map_pattern_inplace");
-    if (guard_rows < 16)
-        return fail(DKV_ERR_INVALID_ARG, "guard_rows=%d < 16: decode reads whole 16-row tiles past a slab's last row",
-                    guard_rows);
+    if (guard_rows < dkv::kMinGuardRows)
+        return fail(DKV_ERR_INVALID_ARG, "guard_rows=%d < %d: decode reads whole %d-row boxes past a slab's last row",
+                    guard_rows, dkv::kMinGuardRows, dkv::kBoxRows);
     const int64_t NH = (int64_t)p->s.L * p->B * p->s.H_kv;
     const int64_t need = NH * p->inplace_stride * dkv::kRowBytes;
     if (dkv::vmm_bytes(m) < need)

@@ -41,7 +41,8 @@
 namespace dkv {
 namespace {
 
-constexpr int kMmaTR = 16;                // rows per tile: the m16 of the score product
+constexpr int kMmaTR = kBoxRows;          // rows per tile: the m16 of the score product, one TMA box
+static_assert(kMmaTR == 16, "m16n8k16");
 constexpr int kBoxBytes = kMmaTR * 128;   // one TMA box: 16 rows x 64 bf16 dims
 constexpr int kHalfTile = 2 * kBoxBytes;  // the K (or V) rows of a tile: dims 0-63, then dims 64-127
 

@@ -11,7 +11,8 @@
 //
 //   warp 0              (one lane issues) TMA: a tile's K rows and V rows, each as 16-row 2-D
 //                       boxes (64 dims, 128-byte swizzle; measured faster than
-//                       64- or 32-row boxes), into separate
+//                       64- or 32-row boxes), only those with rows of the
+//                       segment, into separate
 //                       rings (4 K stages, 5 V stages): a K stage is released as
 //                       soon as its score product is done, a V stage only after
 //                       its output product, so V is the deeper ring.
@@ -80,7 +81,8 @@ constexpr int kTcRows = 64;                    // cache rows per tile
 constexpr int kKStages = 4;                    // K ring stages
 constexpr int kVStages = 5;                    // V ring stages
 constexpr int kTcBox = kTcRows * 128;          // one 64-dim half of a tile: 64 rows x 64 dims of bf16 (8 KB)
-constexpr int kTcBoxRows = 16;                 // rows of one TMA box (measured: 16-row boxes beat 64- and 32-row ones)
+constexpr int kTcBoxRows = kBoxRows;           // rows of one TMA box (measured: 16-row boxes beat 64- and 32-row ones)
+constexpr int kTcBoxPair = 2 * kTcBoxRows * 128;  // both 64-dim halves of one box's rows
 constexpr int kTcHalfTile = 2 * kTcBox;        // K (or V) rows of one tile: dims 0-63, then 64-127
 constexpr int kTcThreads = 320;                // warps: 0 TMA, 1 MMA, 2-5 and 6-9 the two softmax groups
 constexpr int kTcSoft = 256;                   // threads of the softmax warps
@@ -91,6 +93,16 @@ constexpr int kTcQBytes = 2 * kTcQHalf;        // Q as the A operand: 64 rows x 
 constexpr int kTcPBytes = 2 * kTcMaxCols * 128;  // one P buffer: high parts (rows 0..NCpad-1), then low parts, 64 rows each
 constexpr int kTcPre = 1;                      // tiles a CTA fetches before waiting for the previous kernel
 constexpr int kSBufs = 4;                      // TMEM score buffers
+// A tile's boxes past its segment are not fetched (dkv_vmm_trim may have unmapped their
+// rows): their K rows in the stage are those of an earlier tile, whose scores are
+// masked, and their V rows are zeroed like every V row past the segment.
+__host__ __device__ constexpr bool tc_reads_within_guard()
+{
+    for (int cnt = 1; cnt <= kTcRows; ++cnt)
+        if (boxes_of(cnt) * kTcBoxRows - cnt >= kMinGuardRows || boxes_of(cnt) > kTcRows / kTcBoxRows) return false;
+    return true;
+}
+static_assert(tc_reads_within_guard(), "no tile reads further past its segment than the guard rows");
 static_assert((kKStages & (kKStages - 1)) == 0 && (kSBufs & (kSBufs - 1)) == 0, "indexed by masks");
 constexpr int kTcTmemCols = 512;               // S buffers at columns 0, 64, 128, 192; O of group g at 256 + 128 g
 constexpr int kTcOCols = 2 * kTcMaxCols;       // O of one group: the product with P's high parts, then with its low parts
@@ -625,14 +637,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         waited = true;
                     }
                     const int s = tk % kKStages, row = wk.cache_row();
+                    const int boxes = boxes_of(wk.cnt());  // those that hold rows of the segment
                     // Bounds-checked build: the tile's rows lie in the cache (TMA reads
                     // zeros past the end, so the copy stays in bounds either way).
                     in_bounds(row >= 0 && (a.rows_cap == 0 || row + wk.cnt() <= a.rows_cap), a.status);
                     const uint32_t bar = smem_u32(&k_full[s]), dst = smem_u32(ringK + s * kTcHalfTile);
                     if (leads) {
-                        mbar_arrive_expect_tx(bar, kTcHalfTile);
+                        mbar_arrive_expect_tx(bar, boxes * kTcBoxPair);
 #pragma unroll
                         for (int j = 0; j < kTcRows / kTcBoxRows; ++j) {
+                            if (j >= boxes) break;
                             tma_box(dst + j * kTcBoxRows * 128, &maps.k, 0, row + j * kTcBoxRows, bar, pol);
                             tma_box(dst + kTcBox + j * kTcBoxRows * 128, &maps.k, 64, row + j * kTcBoxRows, bar, pol);
                         }
@@ -642,12 +656,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     moved = true;
                 }
                 if (wv.more() && tv < tk && (tv < kVStages || test_phase_warp(&v_empty[tv % kVStages], ((tv / kVStages) - 1) & 1))) {
-                    const int s = tv % kVStages, row = wv.cache_row();
+                    const int s = tv % kVStages, row = wv.cache_row(), boxes = boxes_of(wv.cnt());
                     const uint32_t bar = smem_u32(&v_full[s]), dst = smem_u32(ringV + s * kTcHalfTile);
                     if (leads) {
-                        mbar_arrive_expect_tx(bar, kTcHalfTile);
+                        mbar_arrive_expect_tx(bar, boxes * kTcBoxPair);
 #pragma unroll
                         for (int j = 0; j < kTcRows / kTcBoxRows; ++j) {
+                            if (j >= boxes) break;
                             tma_box(dst + j * kTcBoxRows * 128, &maps.v, 0, row + j * kTcBoxRows, bar, pol);
                             tma_box(dst + kTcBox + j * kTcBoxRows * 128, &maps.v, 64, row + j * kTcBoxRows, bar, pol);
                         }

@@ -11,6 +11,14 @@ namespace dkv {
 constexpr int kHeadDim = 128;   // elements per row
 constexpr int kRowBytes = 256;  // bytes per bf16 row
 
+// The tensor-core decode kernels fetch cache rows in whole TMA boxes of kBoxRows rows
+// from a segment's first row on, so they read up to kBoxRows - 1 rows past its last
+// one. Page-backed buffers keep that many rows mapped behind every slab
+// (dkv_vmm_trim): no kernel may fetch a box that holds none of the segment's rows.
+constexpr int kBoxRows = 16;
+__host__ __device__ constexpr int boxes_of(int rows) { return (rows + kBoxRows - 1) / kBoxRows; }
+constexpr int kMinGuardRows = kBoxRows;
+
 // Bounds-checked build (-DDKV_DEBUG, build.build_library(debug=True)): the
 // kernels check the indices and offsets they read against the ranges the plan
 // gives them, skip an access that falls outside, and set DKV_DEV_BOUNDS in the

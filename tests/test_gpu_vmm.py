@@ -80,3 +80,52 @@ def test_trim_releases_pages_and_decode_still_matches(cuda):
     finally:
         bufK.close()
         bufV.close()
+
+
+@pytest.mark.parametrize("reserve,napp", [(0, 0), (8, 8)])
+@pytest.mark.parametrize("G,Qs", [(4, (1, 2, 4, 5, 16)), (7, (4, 9))])
+def test_multi_query_on_a_trimmed_buffer(cuda, G, Qs, reserve, napp):
+    """Every multi-query kernel on slabs whose last row is the guard's 16 rows short
+    of a page boundary, with the next page released: the 64-row tiles of the
+    17-to-64-column kernel may fetch no 16-row box past a slab's last row."""
+    Hkv, T_stride, guard = 2, 16384, 16
+    buf = [dkv.VmmBuffer(Hkv * T_stride * 256) for _ in range(2)]
+    try:
+        page_rows = buf[0].page_bytes() // 256
+        assert T_stride % page_rows == 0
+        T = page_rows - guard - reserve
+        assert 0 < T and page_rows <= T_stride // 2
+        w = I.Workload("vmm-multi", L=1, H=G * Hkv, Hkv=Hkv, T=T, B=1, D=2, W=T, pattern="ones", rate=1.0, seed=67)
+        M, Tc = I.make_pattern(w), I.context_lengths(w)
+        sh, geo = shapes(w)
+        K, V = (b.tensor((1, 1, Hkv, T_stride, 128), torch.bfloat16) for b in buf)
+        Kh, Vh = I.dense_kv(w.with_(T=T_stride))
+        K.copy_(Kh.to(cuda))
+        V.copy_(Vh.to(cuda))
+        om = O.map_pattern(M, Tc, geo, reserve=reserve)
+        im = O.Mapping(om.len, np.arange(Hkv + 1, dtype=np.int64) * T_stride, om.ioff, om.idx)
+        plan = dkv.dkv_map_pattern_inplace(M, Tc, sh, T_stride, reserve_rows=reserve)
+        dkv.dkv_compact_inplace(plan, K, V)
+        torch.cuda.synchronize()
+        for b in buf:
+            b.trim(plan, guard_rows=guard)
+            # one page a slab is left, exactly the slab's rows, the reserve and the guard
+            assert b.mapped_bytes() == Hkv * b.page_bytes()
+        oKc, oVc = Kh.reshape(-1, 128), Vh.reshape(-1, 128)  # every position is kept, in place
+        n_app = torch.full((1,), napp, dtype=torch.int32, device=cuda)
+        gen = torch.Generator().manual_seed(G)
+        for Q in Qs:
+            q = torch.randn((1, Q, w.H, 128), generator=gen).to(torch.bfloat16)
+            out = torch.full((1, Q, w.H, 128), float("nan"), device=cuda)
+            dkv.dkv_decode_multi(plan, 0, q.to(cuda), Q, n_app, K.reshape(-1, 128), V.reshape(-1, 128), out)
+            got = out.double().cpu().numpy()
+            for i in sorted({0, Q // 2, Q - 1}):
+                want = O.decode(im, 0, 1, w.H, Hkv, I.bf16_bits(q[:, i].contiguous()), I.bf16_bits(oKc),
+                                I.bf16_bits(oVc), n_rows_app=np.full(1, napp, np.int32))
+                assert_close(np.ascontiguousarray(got[:, i]), want, f"Q {Q} query {i}")
+        assert dkv.dkv_plan_status(plan) == 0
+        plan.close()
+        del K, V
+    finally:
+        for b in buf:
+            b.close()
