@@ -243,11 +243,15 @@ void dkv_vmm_free(dkv_vmm* buffer);
  * ordered (same stream, or synchronised). An append past the reserve is skipped
  * and sets DKV_DEV_APPEND_OVERFLOW.
  * The kernels use programmatic dependent launch: they may start while the
- * previous kernel in the stream is still running, and read q, k_new, v_new only
- * after it has completed. n_appended and the packed cache rows of earlier steps
- * are read before that point, so they must not be written by the kernel that
- * immediately precedes this call if that kernel signals early completion
- * (griddepcontrol.launch_dependents); an ordinary kernel never does.
+ * previous kernel in the stream is still running. Until it has completed they
+ * read only the plan, n_appended and the context rows of the cache (the first
+ * len[h] rows of a slab); appended rows, q, k_new and v_new are read afterwards.
+ * So n_appended and the context rows must not be written by a kernel that
+ * signals early completion (griddepcontrol.launch_dependents) unless an ordinary
+ * kernel or a copy lies between it and this call. Of this library the decode
+ * calls and dkv_topk_mask signal early; they write neither, so calls of this
+ * library may follow each other in any order (an append may be followed directly
+ * by a call whose n_appended counts the appended row).
  * Errors: DKV_ERR_INVALID_ARG (NULL/unaligned pointer, layer out of range,
  * only one of k_new/v_new), DKV_ERR_CUDA.
  */

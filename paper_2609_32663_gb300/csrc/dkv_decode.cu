@@ -422,18 +422,23 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const __g
         // computing, drains its copies in flight, and leaves its partials unwritten.
         bool dead = false;
         int inflight = 0;
+        int pre = 0;
 #pragma unroll 1
-        for (int s = 0; s < PRE && ld.h < hend; ++s) {
-            if (lane == 0) issue(ld, s);
+        for (; pre < PRE && ld.h < hend; ++pre) {
+            const int x1 = min(ld.x + TR, ld.s1), b = ld.h / a.Hkv;
+            if (uniform(settled_rows(tab.NA[b], tab.NP[b + 1] - tab.NP[b], ld.x, x1, ld.p0 + ld.n_h)) < x1 - ld.x) break;
+            if (lane == 0) issue(ld, pre);
             ++inflight;
             cursor_next<TR>(ld, a, tab, hend, wA, wB);
         }
-        // Everything above reads only the plan, n_appended and the cache rows of
-        // earlier steps; q, k_new, v_new, the cache slots written here and the
-        // workspace belong to the previous kernel's epoch.
+        // Everything above reads only the plan, n_appended and context rows; rows
+        // appended by earlier calls, q, k_new, v_new, the cache slots written here and
+        // the workspace belong to the previous kernel's epoch. (This kernel signals its
+        // dependents before its own wait, so several kernels back may still be storing
+        // their rows.)
         pdl_wait();
 #pragma unroll 1
-        for (int s = PRE; s < NS && ld.h < hend; ++s) {
+        for (int s = pre; s < NS && ld.h < hend; ++s) {
             if (lane == 0) issue(ld, s);
             ++inflight;
             cursor_next<TR>(ld, a, tab, hend, wA, wB);

@@ -254,7 +254,21 @@ struct Segment {
     int row;    // cache row of the first of them
     int p0, p1; // the slab's layer rows
     int app;    // the segment's last row is this step's new token
+    int settled; // of the segment's rows, from the first, those that the wait need not precede
 };
+
+// How many of the layer rows [s0, s1) of a slab that ends at p1, from s0 on, may be
+// fetched before the wait for the previous kernel: all of them if no earlier call
+// appended to the slab (na rows), else those of the context (all but the extra rows at
+// its end). An earlier decode call lets the next kernel start before its appended row
+// is stored, so such rows are fetched only after the wait. (This call's own new row
+// comes from k_new and v_new.)
+__device__ __forceinline__ int settled_rows(int na, int extra, int s0, int s1, int p1)
+{
+    return na > 0 ? max(0, min(s1, p1 - extra) - s0) : s1 - s0;
+}
+
+constexpr int kSegmentWords = 8;  // of a warp's segment slot (7 used)
 
 // The first segment of a slab in [h, hend), which has one, of a warp with the
 // layer rows [wA, wB), into the warp's slot in shared memory. (Returned that way,
@@ -272,21 +286,25 @@ __device__ __noinline__ void find_segment(const DecodeArgs& a, unsigned char* ta
         if (max(wA, p0) < min(wB, p1)) break;
     }
     const int s0 = max(wA, p0), s1 = min(wB, p1), b = h / a.Hkv;
+    const int na = t.NA[b], extra = t.NP[b + 1] - t.NP[b];
+    const int64_t off = t.OFF ? t.OFF[h] : a.off[h];
     __syncwarp();
     if ((threadIdx.x & 31) == 0) {
         slot[0] = h;
         slot[1] = s1 - s0;
-        slot[2] = (int)((t.OFF ? t.OFF[h] : a.off[h]) + (s0 - p0));
+        slot[2] = (int)(off + (s0 - p0));
         slot[3] = p0;
         slot[4] = p1;
-        slot[5] = (a.append && s1 == p1 && t.NP[b + 1] - t.NP[b] > t.NA[b]) ? 1 : 0;
+        slot[5] = (a.append && s1 == p1 && extra > na) ? 1 : 0;
+        slot[6] = settled_rows(na, extra, s0, s1, p1);
     }
     __syncwarp();
 }
 
 __device__ __forceinline__ Segment read_segment(const int32_t* slot)
 {
-    return {uniform(slot[0]), uniform(slot[1]), uniform(slot[2]), uniform(slot[3]), uniform(slot[4]), uniform(slot[5])};
+    return {uniform(slot[0]), uniform(slot[1]), uniform(slot[2]), uniform(slot[3]), uniform(slot[4]), uniform(slot[5]),
+            uniform(slot[6])};
 }
 
 // Slabs of the warp's first and last row.

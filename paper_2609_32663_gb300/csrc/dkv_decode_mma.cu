@@ -52,7 +52,7 @@ struct MK {
     static constexpr int kWarpRing = NS * kHalfTile;
     static constexpr int kRingBytes = NW * kWarpRing;
     static constexpr int kBarBytes = NW * NS * 8;
-    static constexpr int kMetaBytes = (TailMeta<NW>::kWords + 8 * NW) * 4;  // and a segment slot a warp
+    static constexpr int kMetaBytes = (TailMeta<NW>::kWords + kSegmentWords * NW) * 4;  // and a segment slot a warp
     static constexpr int kDepOff = (8 * NT * (kHeadDim + 2) * 4 + 15) / 16 * 16;  // after a warp's final state
     static constexpr int kAlign = 1024;                  // swizzle atoms are 1024-byte aligned
     static constexpr int kFixedBytes = kRingBytes + kBarBytes + kMetaBytes;
@@ -429,6 +429,7 @@ __global__ void __launch_bounds__(MKFor<G, NT, MULTI>::NW * 32, 1)
     // merge, and fill the memory pipe while it runs (us per step with 2, 3, 4: 128K
     // 1,018 / 1,007 / 1,033, 32K 425 / 423 / 461, ragged batch of 16 662 / 655 / 656).
     constexpr int NPRE = NS < 3 ? NS : 3;
+    static_assert(NPRE <= 3, "the first two tiles are checked for rows that an earlier call appends");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // The ring starts on a 1024-byte boundary (the swizzle pattern's period).
     unsigned char* smem = smem_raw + ((C::kAlign - (smem_u32(smem_raw) & (C::kAlign - 1))) & (C::kAlign - 1));
@@ -482,7 +483,7 @@ __global__ void __launch_bounds__(MKFor<G, NT, MULTI>::NW * 32, 1)
         const int2 hr = slab_range(a, table, wA, wB);
         const int hfirst = uniform(hr.x), hlast = uniform(hr.y);
         const uint64_t pol = evict_first_policy();
-        int32_t* slot = meta + TM::kWords + 8 * warp;
+        int32_t* slot = meta + TM::kWords + kSegmentWords * warp;
         find_segment(a, table, hfirst, hlast + 1, wA, wB, slot);
         Segment cp = read_segment(slot);  // the segment being computed; `left` and `row` run on tile by tile
         int ld_h = cp.h, ld_left = cp.left, ld_row = cp.row;  // the next tile to fetch
@@ -526,15 +527,22 @@ __global__ void __launch_bounds__(MKFor<G, NT, MULTI>::NW * 32, 1)
         // A bounded wait that runs out marks the warp dead: it stops issuing and
         // computing, drains its copies in flight, and leaves its partials unwritten.
         bool dead = false;
+        // Before the wait, only tiles of settled rows (K0 V0 K1: the first two tiles).
+        const int whole = cp.settled >= cp.left ? NPRE : 2 * (cp.settled / TR);
+        int pre = 0;
 #pragma unroll 1
-        for (int s = 0; s < NPRE; ++s) issue_next();
-        // Everything above reads only the plan, n_appended and the cache rows of
-        // earlier steps; q, k_new, v_new, the cache slots written here and the
-        // workspace belong to the previous kernel's epoch.
+        for (; pre < min(NPRE, whole); ++pre) {
+            // A second tile of another segment, which is then the one in the slot.
+            if (pre == 2 && cp.left <= TR && uniform(slot[6]) < min(TR, ld_left)) break;
+            issue_next();
+        }
+        // Everything above reads only the plan, n_appended and context rows; rows
+        // appended by earlier calls, q, k_new, v_new, the cache slots written here and
+        // the workspace belong to the previous kernel's epoch.
         pdl_wait();
         pdl_launch_dependents();  // only now: the next kernel may then rely on everything before this one
 #pragma unroll 1
-        for (int s = NPRE; s < NS; ++s) issue_next();
+        for (int s = pre; s < NS; ++s) issue_next();
         int stage = 0;
         uint32_t phase = 0;
         const float cs = a.qscale;  // softmax scale * log2(e)

@@ -92,6 +92,7 @@ constexpr int kTcQHalf = kTcQRows * 128;       // one 64-dim half of Q (8 KB)
 constexpr int kTcQBytes = 2 * kTcQHalf;        // Q as the A operand: 64 rows x 128 dims (two buffers: segments alternate)
 constexpr int kTcPBytes = 2 * kTcMaxCols * 128;  // one P buffer: high parts (rows 0..NCpad-1), then low parts, 64 rows each
 constexpr int kTcPre = 1;                      // tiles a CTA fetches before waiting for the previous kernel
+static_assert(kTcPre == 1, "only the first tile is checked for rows that an earlier call appends");
 constexpr int kSBufs = 4;                      // TMEM score buffers
 // A tile's boxes past its segment are not fetched (dkv_vmm_trim may have unmapped their
 // rows): their K rows in the stage are those of an earlier tile, whose scores are
@@ -123,8 +124,8 @@ constexpr int kNumBars = 2 * kKStages + 2 * kVStages + kSBufs + 7;
 constexpr int kOffTmem = kOffBars + kNumBars * 8;
 constexpr int kOffInfo = kOffTmem + 16;                   // int[kInfoWords]: the CTA's share (TcShare)
 constexpr int kInfoWords = 8;
-constexpr int kOffSlots = kOffInfo + kInfoWords * 4;      // int[6] a warp: its current segment
-constexpr int kOffTable = (kOffSlots + kTcThreads / 32 * 24 + 15) / 16 * 16;
+constexpr int kOffSlots = kOffInfo + kInfoWords * 4;      // int[kSegmentWords] a warp: its current segment
+constexpr int kOffTable = (kOffSlots + kTcThreads / 32 * kSegmentWords * 4 + 15) / 16 * 16;
 constexpr int kTcAlign = 1024;
 __host__ __device__ constexpr int tc_smem_bytes(int B) { return kTcAlign + kOffTable + seq_table_bytes(B); }
 static_assert(tc_smem_bytes(kMaxB) <= 227 * 1024, "fits the opt-in shared memory of one CTA");
@@ -608,7 +609,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         return;
     }
     const int hfirst = uniform(share->hfirst), hend = uniform(share->hlast) + 1;
-    int32_t* slot = reinterpret_cast<int32_t*>(sm + kOffSlots) + 6 * warp;
+    int32_t* slot = reinterpret_cast<int32_t*>(sm + kOffSlots) + kSegmentWords * warp;
     const int NC = a.NC;
     const int NCpad = (NC + 15) & ~15;
     const float cs = a.qscale;
@@ -625,6 +626,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             TileWalk wk, wv;
             wk.begin(a, table, hfirst, hend, A, Bc, slot);
             wv = wk;
+            // The first tile is fetched before the wait only if all its rows are settled.
+            const bool early = wk.sg.settled >= wk.cnt();
             int tk = 0, tv = 0;
             bool waited = false;
             IdleBound idle;
@@ -632,7 +635,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             while ((wk.more() || wv.more()) && !uniform(flags[kFlagAbort])) {
                 bool moved = false;
                 if (wk.more() && (tk < kKStages || test_phase_warp(&k_empty[tk % kKStages], ((tk / kKStages) - 1) & 1))) {
-                    if (tk == kTcPre && !waited) {
+                    if ((tk == kTcPre || !early) && !waited) {
                         pdl_wait();  // later copies after the previous kernel, as in the other kernels
                         waited = true;
                     }
