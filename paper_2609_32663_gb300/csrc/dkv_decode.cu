@@ -375,7 +375,10 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const __g
     }
     const int P = live_parts(R, a.nctas);  // CTAs with rows
     const int A = c < P ? part_start(c, R, P) : R, Bc = c < P ? part_start(c + 1, R, P) : R;
-    if (A >= Bc) return;  // uniform: this CTA has no rows
+    if (A >= Bc) {  // uniform: this CTA has no rows
+        pdl_wait();  // so that the grid does not complete before the previous kernel has
+        return;
+    }
     const int wA = A + (int)(((int64_t)(Bc - A) * warp) / NW);
     const int wB = A + (int)(((int64_t)(Bc - A) * (warp + 1)) / NW);
     unsigned char* my_ring = smem + warp * NS * C::kStageBytes;

@@ -105,3 +105,18 @@ def test_allocation_free_appends_in_a_row(G, T):
     r.check_appends()
     assert status.item() == 0
     c.close()
+
+
+def test_allocation_free_call_without_rows_waits_for_the_one_before():
+    """A layer with no rows: its zeros are written after the previous call's outputs."""
+    r = Run(4, 30000)
+    c, w, info = r.c, r.c.wl, r.c.info
+    none = torch.zeros(w.B * w.Hkv + 1, dtype=torch.int64, device=c.dev)
+    out = torch.full((20, w.B, w.H, 128), float("nan"), device=c.dev)
+    torch.cuda.synchronize()
+    for o in out:
+        dkv.dkv_decode_attn_noalloc(c.sh, w.B, 0, c.reserve, info.d_len, info.d_off, info.d_ioff, r.dq[0], None, None,
+                                    None, c.Kc, c.Vc, o)
+        dkv.dkv_decode_attn_noalloc(c.sh, w.B, 0, c.reserve, none, none, none, r.dq[0], None, None, None, c.Kc, c.Vc, o)
+    assert not out.any()
+    c.close()
