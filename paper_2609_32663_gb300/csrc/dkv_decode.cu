@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const __g
                 const uint16_t* qrow = a.q + ((int64_t)b * a.H + g * G + j) * kHeadDim;
 #pragma unroll
                 for (int i = 0; i < NCH; ++i)
-                    bf8_to_f2x4(__ldg(reinterpret_cast<const uint4*>(qrow + 8 * (sl + LPR * i))), q2[j] + 4 * i);
+                    bf8_to_f2x4(ld_prev(reinterpret_cast<const uint4*>(qrow + 8 * (sl + LPR * i))), q2[j] + 4 * i);
             }
 #pragma unroll
             for (int j = 0; j < G; ++j) {
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(C::NW * 32, 1) decode_partial_kernel(const __g
                     // slab's next free row for later steps.
                     const int half = lane >> 4, sub = lane & 15;
                     const uint16_t* src = (half ? a.v_new : a.k_new) + ((int64_t)b * a.Hkv + g) * kHeadDim;
-                    const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + sub);
+                    const uint4 v = ld_prev(reinterpret_cast<const uint4*>(src) + sub);
                     *reinterpret_cast<uint4*>((half ? vt : kt) + (cnt - 1) * kRowBytes + sub * 16) = v;
                     const int64_t nrow = cp.base + (cp.n_h - 1);
                     if (in_bounds(nrow >= 0 && (a.rows_cap == 0 || nrow < a.rows_cap), a.status)) {

@@ -191,8 +191,8 @@ __device__ __forceinline__ void load_q(const DecodeArgs& a, int b, int g, int NC
             reinterpret_cast<const uint32_t*>(a.q + (live ? ((int64_t)b * a.Q + qi) * a.H + g * G + j : 0) * kHeadDim);
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
-            qb[nt][kk][0] = live ? __ldg(qr + 8 * kk + t) : 0u;
-            qb[nt][kk][1] = live ? __ldg(qr + 8 * kk + t + 4) : 0u;
+            qb[nt][kk][0] = live ? ld_prev(qr + 8 * kk + t) : 0u;
+            qb[nt][kk][1] = live ? ld_prev(qr + 8 * kk + t + 4) : 0u;
         }
     }
 }
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(MKFor<G, NT, MULTI>::NW * 32, 1)
             // round trips there held up every slab by 1.4 us).
             uint4 fresh_row = make_uint4(0u, 0u, 0u, 0u);
             if (cp.app)
-                fresh_row = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? a.k_new : a.v_new) +
+                fresh_row = ld_prev(reinterpret_cast<const uint4*>((lane < 16 ? a.k_new : a.v_new) +
                                                                  ((int64_t)b * a.Hkv + g) * kHeadDim) + (lane & 15));
             state_reset(S);
             if (prefetch) {

@@ -385,7 +385,7 @@ __device__ void load_q_tc(const DecodeArgs& a, int h, unsigned char* sQ, int tid
         v[u] = make_uint4(0u, 0u, 0u, 0u);
         if (c < a.NC) {
             const int qi = c / G, j = c - qi * G;
-            v[u] = __ldg(reinterpret_cast<const uint4*>(a.q + (((int64_t)b * a.Q + qi) * a.H + g * G + j) * kHeadDim) + ch);
+            v[u] = ld_prev(reinterpret_cast<const uint4*>(a.q + (((int64_t)b * a.Q + qi) * a.H + g * G + j) * kHeadDim) + ch);
         }
     }
 #pragma unroll

@@ -72,6 +72,37 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
     return mbar_try_wait(bar, parity) || mbar_wait_more(bar, parity);
 }
 
+// Loads of what the previous kernel in the stream may write (after griddepcontrol.wait).
+// Not __ldg: a non-coherent load is for data that nothing writes while the kernel runs,
+// and a kernel that starts before the previous one has ended does run meanwhile.
+__device__ __forceinline__ uint4 ld_prev(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ float4 ld_prev(const float4* p)
+{
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ uint32_t ld_prev(const uint32_t* p)
+{
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ float ld_prev(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ uint64_t evict_first_policy()
 {
     uint64_t pol;

@@ -23,6 +23,7 @@
 // are long), and a CTA adds its nonzero bins to the global histogram.
 #include "dkv.h"
 #include "dkv_internal.cuh"
+#include "dkv_ptx.cuh"
 
 #include <cooperative_groups.h>
 
@@ -325,12 +326,12 @@ __global__ void __launch_bounds__(kClThreads, 1) topk_cluster_kernel(const float
         const int i = wlo + kClUnit * u;
         v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (vec_p && i + 3 < whi) {
-            v[u] = __ldg(reinterpret_cast<const float4*>(P + i));
+            v[u] = ld_prev(reinterpret_cast<const float4*>(P + i));
         } else {
-            if (i < whi) v[u].x = __ldg(P + i);
-            if (i + 1 < whi) v[u].y = __ldg(P + i + 1);
-            if (i + 2 < whi) v[u].z = __ldg(P + i + 2);
-            if (i + 3 < whi) v[u].w = __ldg(P + i + 3);
+            if (i < whi) v[u].x = ld_prev(P + i);
+            if (i + 1 < whi) v[u].y = ld_prev(P + i + 1);
+            if (i + 2 < whi) v[u].z = ld_prev(P + i + 2);
+            if (i + 3 < whi) v[u].w = ld_prev(P + i + 3);
         }
     }
     uint32_t key[KPT];

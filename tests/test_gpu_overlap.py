@@ -120,3 +120,24 @@ def test_allocation_free_call_without_rows_waits_for_the_one_before():
         dkv.dkv_decode_attn_noalloc(c.sh, w.B, 0, c.reserve, none, none, none, r.dq[0], None, None, None, c.Kc, c.Vc, o)
     assert not out.any()
     c.close()
+
+
+@pytest.mark.parametrize("T", [1200, 30000])
+def test_export_of_what_the_previous_call_writes(T):
+    """A decode call signals early; the export that follows reads its outputs as
+    probabilities, in one buffer that every step rewrites."""
+    r = Run(4, T)
+    c, w = r.c, r.c.wl
+    n = w.B * w.H * 128
+    P = torch.full((w.B, w.H, 128), float("nan"), device=c.dev)
+    kept = torch.empty_like(P).expand(STEPS, *P.shape).clone()
+    M = torch.full((STEPS, n), 7, dtype=torch.uint8, device=c.dev)
+    work = torch.empty(dkv.dkv_topk_workspace_bytes(), dtype=torch.uint8, device=c.dev)
+    torch.cuda.synchronize()
+    for s in range(STEPS):
+        dkv.dkv_decode_attn(c.plan, 0, r.dq[s], None, None, None, c.Kc, c.Vc, P)
+        dkv.dkv_topk_mask(P, n // 3, M[s], work)
+        dkv.dkv_decode_attn(c.plan, 0, r.dq[s], None, None, None, c.Kc, c.Vc, kept[s])
+    for s in range(STEPS):
+        assert np.array_equal(M[s].cpu().numpy(), O.topk_mask(kept[s].cpu().numpy(), n // 3).reshape(-1)), f"step {s}"
+    c.close()
