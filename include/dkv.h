@@ -59,7 +59,7 @@ typedef enum {
 /* Device status word bits (dkv_plan_status). */
 #define DKV_DEV_APPEND_OVERFLOW 0x1 /* n_appended reached the slab's reserve: token not appended */
 #define DKV_DEV_TMA_TIMEOUT 0x2     /* a bulk copy did not complete within the wait bound */
-#define DKV_DEV_MERGE_TIMEOUT 0x4   /* a fused merge's partials were not all written within the wait bound */
+#define DKV_DEV_MERGE_TIMEOUT 0x4   /* a fused merge's partials were not all written within the wait bound: outputs of the plan's calls are not to be used until the word is cleared */
 #define DKV_DEV_BOUNDS 0x8          /* bounds-checked build only: an index or offset a kernel read was out of its range; the access was skipped */
 
 /* Pattern and model geometry (Sec. 3.2, Sec. 3.4). */
@@ -312,7 +312,10 @@ dkv_status dkv_advance(const dkv_plan* plan, int32_t* n_appended, cudaStream_t s
 
 /*
  * Read (and optionally clear) the plan's device status word (DKV_DEV_* bits).
- * Synchronises `stream`. Returns DKV_OK even when bits are set.
+ * Synchronises `stream`. Returns DKV_OK even when bits are set. A merge that gave
+ * up (DKV_DEV_MERGE_TIMEOUT) can leave a partial result in the plan, which the next
+ * call may take for its own: clearing the word removes it (no call of the plan may
+ * be running on another stream then).
  */
 dkv_status dkv_plan_status(const dkv_plan* plan, int32_t* word, int32_t clear, cudaStream_t stream);
 

@@ -78,7 +78,9 @@ dkv_status ok()
 // kernel then sets DKV_DEV_TMA_TIMEOUT and returns; nothing faults),
 // DKV_FAULT=merge makes the last CTA of each fused merge wait for one partial
 // more than the slab has (the wait runs out, sets DKV_DEV_MERGE_TIMEOUT and
-// skips that merge), and DKV_FAULT=barrier makes the Top-K export's grid
+// skips that merge), DKV_FAULT=late leaves every exchange word full after a decode
+// step, with the same status bit, as partials do that arrive after their merge gave up,
+// and DKV_FAULT=barrier makes the Top-K export's grid
 // barriers wait for a CTA that does not exist (the first wait runs out and sets
 // the workspace status word).
 bool fault(const char* what)
@@ -719,6 +721,11 @@ dkv_status dkv_decode_attn(const dkv_plan* p, int32_t layer, const void* q, cons
                                 true, true, &a);
     if (st != DKV_OK) return st;
     st = launch_split_k(p, a, true, stream);
+    if (st == DKV_OK && fault("late")) {
+        const cudaError_t e = cudaMemsetAsync(p->d_exch, 0x40, (size_t)exch_floats(p) * sizeof(float), stream);
+        if (e != cudaSuccess || cudaMemsetAsync(p->d_status, DKV_DEV_MERGE_TIMEOUT, 1, stream) != cudaSuccess)
+            return fail(DKV_ERR_CUDA, "injected late partials: memset failed");
+    }
     return st == DKV_OK ? ok() : st;
 }
 
@@ -818,6 +825,13 @@ dkv_status dkv_plan_status(const dkv_plan* p, int32_t* word, int32_t clear, cuda
     if ((e = cudaMemcpyAsync(word, p->d_status, 4, cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(stream)) != cudaSuccess)
         return cuda_fail(e, "read status word");
+    if (clear && (*word & DKV_DEV_MERGE_TIMEOUT)) {
+        // A partial that came after its merge had given up is still in the exchange, where
+        // the next launch would take it for its own. Its writer has ended (the wait above).
+        if ((e = cudaMemsetAsync(p->d_exch, 0, (size_t)exch_floats(p) * sizeof(float), stream)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(stream)) != cudaSuccess)
+            return cuda_fail(e, "clear exchange");
+    }
     if (clear && (e = cudaMemsetAsync(p->d_status, 0, 4, stream)) != cudaSuccess) return cuda_fail(e, "clear status");
     return ok();
 }

@@ -353,7 +353,12 @@ __device__ __forceinline__ void write_out(const DecodeArgs& a, int b, int g, int
 // then the loads: at 32K (50 MB layers) 9.3 us of streaming was followed by up
 // to 5.1 us of merge, now 3.3. The merging CTA empties the slots again for the
 // next launch (ordered by the launches' dependency). It waits only for CTAs of
-// lower index, which start no later than it does.
+// lower index. Where the device holds the whole grid (one CTA an SM) they all run at
+// once; elsewhere this assumes that CTAs start in the order of their index, as they do
+// but as CUDA does not promise. If that fails the wait runs out: the outputs stay
+// unwritten and the status word says so. A partial that arrives after its merge gave up
+// stays in the exchange until the status word is cleared (dkv_plan_status empties the
+// exchange then): until that, no output of the plan is to be trusted.
 __device__ __forceinline__ float full_word(float x) { return __float_as_uint(x) == 0u ? -0.f : x; }
 
 __device__ __forceinline__ bool is_full(const float4& v)

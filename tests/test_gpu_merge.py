@@ -120,3 +120,28 @@ def test_plans_of_other_sizes_side_by_side():
     big.decode_steps(1, append=False)
     for c in [big] + small:
         c.close()
+
+
+@pytest.mark.parametrize("G,Q", [(4, 1), (7, 1), (4, 2), (4, 4)])
+def test_a_partial_that_came_late_is_gone_after_the_status_is_cleared(monkeypatch, G, Q):
+    """DKV_FAULT=late: every exchange word is full after the call, as if partials had
+    arrived after their merge gave up. Once the status word is cleared, the next call
+    of any kind is exact."""
+    w = wl(L=1, H=2 * G, Hkv=2, T=9000, W=4000, B=2, seed=G)
+    c = Case(w, reserve=4)
+    gen = torch.Generator().manual_seed(G)
+    q = torch.randn((2, Q, 2 * G, 128), generator=gen).to(torch.bfloat16)
+    dq = q.to(c.dev)
+    out = torch.full((2, Q, 2 * G, 128), float("nan"), device=c.dev)
+    scratch = torch.empty((2, 2 * G, 128), device=c.dev)
+    monkeypatch.setenv("DKV_FAULT", "late")
+    dkv.dkv_decode_attn(c.plan, 0, dq[:, 0].contiguous(), None, None, None, c.Kc, c.Vc, scratch)
+    monkeypatch.delenv("DKV_FAULT")
+    assert dkv.dkv_plan_status(c.plan, clear=True) == dkv.DKV_DEV_MERGE_TIMEOUT
+    dkv.dkv_decode_multi(c.plan, 0, dq, Q, None, c.Kc, c.Vc, out)
+    got = out.double().cpu().numpy()
+    for i in sorted({0, Q - 1}):
+        want = O.decode(c.om, 0, 2, 2 * G, 2, I.bf16_bits(q[:, i].contiguous()), c.oKc, c.oVc)
+        assert_close(np.ascontiguousarray(got[:, i]), want, f"query {i}")
+    c.decode_steps(2, append=True)
+    c.close()
