@@ -58,8 +58,8 @@
 // Every wait is bounded (polls and 2 s). A wait that runs out sets a
 // DKV_DEV_* bit, the roles stop (the softmax groups keep walking the tiles,
 // without work, so that they still meet at every named barrier), the copies and
-// products in flight are drained with the same bound, and TMEM is freed before
-// the CTA exits.
+// products in flight are drained with the same bound, TMEM is freed before the CTA
+// exits, and the combine leaves the outputs of the CTA's shared slabs unwritten.
 //
 // What bounds it: a 64-row tile is 32 KB, 0.73 us at an SM's share of HBM, and its
 // products need 0.3 us of the tensor pipe's operand bandwidth, so the schedules of
@@ -548,6 +548,25 @@ __device__ __noinline__ void write_empty_slabs_tc(const DecodeArgs& a, unsigned 
             for (int j = 0; j < a.NC; ++j)
                 write_out<G>(a, h / a.Hkv, h % a.Hkv, j, make_float4(0.f, 0.f, 0.f, 0.f), 0.f, lane);
         }
+}
+
+// What a CTA that gave up a wait leaves for the combine (one warp): its partials of
+// the slabs it shares are marked missing (a sum below 0, which no softmax has), so that
+// their outputs stay unwritten, and its slabs' slab_parts words are this launch's.
+constexpr float kMissing = -1.f;
+__device__ __noinline__ void mark_missing(const DecodeArgs& a, unsigned char* table, int c, const TcShare* share, int lane)
+{
+    const SeqTable t = seq_table_at(table, a);
+#pragma unroll 1
+    for (int h = share->hfirst; h <= share->hlast; ++h) {
+        const int p0 = slab_start(a, t, h);
+        if (p0 == slab_start(a, t, h + 1)) continue;
+        const int n = h == share->hfirst ? share->n_first : h == share->hlast ? share->n_last : 1;
+        if (p0 >= share->A && lane == 0) *reinterpret_cast<int2*>(a.slab_parts + 2 * h) = make_int2(c, n);
+        if (n > 1)
+            for (int j = lane; j < a.NC; j += 32)
+                *reinterpret_cast<float2*>(a.work_ml + (((int64_t)c + h) * a.NC + j) * 2) = make_float2(-INFINITY, kMissing);
+    }
 }
 
 template <int G>
@@ -1122,6 +1141,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             for (int u = max(0, nk - kKStages); u < nk; ++u) wait_phase(&k_full[u % kKStages], (u / kKStages) & 1);
             for (int u = max(0, nv - kVStages); u < nv; ++u) wait_phase(&v_full[u % kVStages], (u / kVStages) & 1);
         }
+        if (warp == 2) mark_missing(a, table, c, share, lane);
         if (warp == 1 && uniform(flags[kFlagMmaLast])) {
             if (elect_one()) {
                 umma_commit(smem_u32(fin));
@@ -1202,6 +1222,7 @@ __global__ void __launch_bounds__(kCombineCols * 32) combine_tc_kernel(const __g
         }
 #pragma unroll
         for (int u = 0; u < KB; ++u) asm volatile("" : "+f"(v[u].x), "+f"(v[u].y), "+f"(v[u].z), "+f"(v[u].w));
+        if (__any_sync(kFull, ml.y < 0.f)) return;  // a CTA gave up (mark_missing)
         float Mn = fmaxf(M, ml.x);
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) Mn = fmaxf(Mn, __shfl_xor_sync(kFull, Mn, o));

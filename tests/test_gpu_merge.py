@@ -145,3 +145,26 @@ def test_a_partial_that_came_late_is_gone_after_the_status_is_cleared(monkeypatc
         assert_close(np.ascontiguousarray(got[:, i]), want, f"query {i}")
     c.decode_steps(2, append=True)
     c.close()
+
+
+@pytest.mark.parametrize("Hkv,B,Q,T", [(2, 2, 5, 9000), (2, 2, 16, 9000), (8, 9, 5, 1800)])
+def test_outputs_of_a_timed_out_multi_query_call_stay_unwritten(monkeypatch, Hkv, B, Q, T):
+    """DKV_FAULT=copy, 17 or more columns, up to and above 64 slabs: the combine
+    kernel writes nothing from the partials that an earlier call left behind."""
+    G = 4
+    c = Case(wl(H=G * Hkv, Hkv=Hkv, B=B, T=T, W=T, seed=Q))
+    gen = torch.Generator().manual_seed(T)
+    q = torch.randn((B, Q, G * Hkv, 128), generator=gen).to(torch.bfloat16).to(c.dev)
+    first, out, again = (torch.full(q.shape, -7.0, device=c.dev) for _ in range(3))
+    dkv.dkv_decode_multi(c.plan, 0, q, Q, None, c.Kc, c.Vc, first)
+    torch.cuda.synchronize()
+    monkeypatch.setenv("DKV_FAULT", "copy")
+    dkv.dkv_decode_multi(c.plan, 0, q, Q, None, c.Kc, c.Vc, out)
+    torch.cuda.synchronize()
+    monkeypatch.delenv("DKV_FAULT")
+    assert dkv.dkv_plan_status(c.plan, clear=True) & dkv.DKV_DEV_TMA_TIMEOUT
+    assert (out == -7.0).all()
+    dkv.dkv_decode_multi(c.plan, 0, q, Q, None, c.Kc, c.Vc, again)
+    assert torch.equal(again, first)
+    assert dkv.dkv_plan_status(c.plan) == 0
+    c.close()
