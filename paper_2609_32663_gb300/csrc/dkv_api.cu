@@ -37,7 +37,7 @@ struct dkv_plan {
     int32_t* d_status = nullptr;
     float* d_work = nullptr;    // split-K partials
     float* d_exch = nullptr;    // exchange of the fused merge: slots x kMaxCols x (128 + 2) words, 0 between launches
-    int64_t exch_slots = 0;     // (CTA, slab) slots of the exchange
+    int64_t exch_slots = 0;     // CTAs of the largest grid: one slot each
     int32_t* d_slab_parts = nullptr;  // [B*H_kv][2] which CTAs hold a slab's partials (tcgen05 kernel)
     dkv::DecodeConfig cfg{};         // the decode step's kernel (cfg_f32 or cfg_mma)
     dkv::DecodeConfig cfg_f32{};     // fp32 kernel (caches of 2^31 rows or more)
@@ -77,8 +77,10 @@ dkv_status ok()
 // half the bytes a stage expects, so every bounded copy wait runs out (the
 // kernel then sets DKV_DEV_TMA_TIMEOUT and returns; nothing faults),
 // DKV_FAULT=merge makes the last CTA of each fused merge wait for one partial
-// more than the slab has (the wait runs out, sets DKV_DEV_MERGE_TIMEOUT and
-// skips that merge), DKV_FAULT=late leaves every exchange word full after a decode
+// more than the slab has, in its own slot (unless that holds its partial of its next
+// slab, whose merge then misses it, the wait runs out, sets DKV_DEV_MERGE_TIMEOUT and
+// skips that merge; multi-query of 17 or more columns merges in a kernel of its own
+// and waits for nothing), DKV_FAULT=late leaves every exchange word full after a decode
 // step, with the same status bit, as partials do that arrive after their merge gave up,
 // and DKV_FAULT=barrier makes the Top-K export's grid
 // barriers wait for a CTA that does not exist (the first wait runs out and sets
@@ -231,7 +233,7 @@ dkv_status plan_configs(dkv_plan* p)
     }
     const int64_t NHl = (int64_t)p->B * p->s.H_kv;
     p->work = dkv::workspace_layout(ctas + NHl, dkv::kTcMaxCols, warp_records, dkv::kMaxCols);
-    p->exch_slots = ctas + NHl;
+    p->exch_slots = ctas;
     return DKV_OK;
 }
 

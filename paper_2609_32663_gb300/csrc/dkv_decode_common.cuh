@@ -344,9 +344,10 @@ __device__ __forceinline__ void write_out(const DecodeArgs& a, int b, int g, int
 
 // ------------------------------------------------------------ cross-CTA merge
 // A slab whose rows lie in several CTAs is merged by the last of them (by index):
-// every other CTA leaves its partial (m, l, o) of a column in the fused-merge
-// exchange, slot c + h, and the merging CTA polls the slots until every word has
-// arrived. A slot's words carry their own arrival: an empty word is 0, and a
+// every other CTA leaves its partial (m, l, o) of a column in its slot of the
+// fused-merge exchange (a CTA leaves one slab's at most: that of its last slab, if rows
+// of it follow in the next CTA), and the merging CTA polls the slots until every word
+// has arrived. A slot's words carry their own arrival: an empty word is 0, and a
 // partial's zeros are written as -0, so a word is data as soon as it differs from
 // 0, whatever order the stores arrive in. That takes one store and one load
 // through L2, where an arrival counter took a fence, an atomic, an acquire and
@@ -405,28 +406,29 @@ __device__ __forceinline__ bool polled_out(int spin, unsigned long long& t0)
     return __any_sync(kFull, spin >= kWaitSpins || now - t0 > kWaitNs);
 }
 
-// One warp writes a CTA's partial of one column: slot index sj = (c + h) NC + j.
-__device__ __forceinline__ void put_partial(const DecodeArgs& a, int64_t sj, float4 O, float M, float L, int lane)
+// One warp writes CTA c's partial of column j.
+__device__ __forceinline__ void put_partial(const DecodeArgs& a, int c, int j, int NC, float4 O, float M, float L, int lane)
 {
+    const int64_t sj = (int64_t)c * NC + j;
     st_exchange4(a.exch_o + sj * kHeadDim + 4 * lane,
                  make_float4(full_word(O.x), full_word(O.y), full_word(O.z), full_word(O.w)));
     if (lane == 0) st_exchange2(a.exch_ml + sj * 2, full_word(M), full_word(L));
 }
 
 // One warp of the merging CTA adds to a state (M, L, O: 4 dims a lane) of column
-// j of slab h the partials of the CTAs first, first + step, ... below end (step 1
+// j of a slab the partials of the CTAs first, first + step, ... below end (step 1
 // or 2), KB at a time, and empties their slots. A batch is one round trip to L2
 // (0.5 us) once its words are there: lane k reads the k-th partial's m and l,
 // every lane its dims of all of them. KB = 12: with 8 a slab of 19 CTAs takes a
 // second round (128K 1,026 -> 1,040 us per step, 4K 261 -> 280), 16 is no faster.
 // False when a partial did not arrive within the wait bound.
 template <int KB, int NCC>
-__device__ __forceinline__ bool merge_partials(const DecodeArgs& a, int h, int j, int NC_, int first, int step,
+__device__ __forceinline__ bool merge_partials(const DecodeArgs& a, int j, int NC_, int first, int step,
                                                int end, float& M, float& L, float4& O, int lane)
 {
     const int NC = NCC ? NCC : NC_;
     const int stride = step * NC;
-    const int64_t base = ((int64_t)first + h) * NC + j;
+    const int64_t base = (int64_t)first * NC + j;
     float* po = a.exch_o + base * kHeadDim + 4 * lane;
     float* pm = a.exch_ml + (base + (int64_t)lane * stride) * 2;
     bool good = true;
@@ -506,9 +508,9 @@ __device__ __noinline__ void dead_tail(const DecodeArgs& a, const SeqTable& tab,
             float M = -INFINITY, L = 0.f;
             float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
             if (c1 == c)
-                merge_partials<4, 0>(a, h, j, NC, c0, 1, c1, M, L, O, lane);
+                merge_partials<4, 0>(a, j, NC, c0, 1, c1, M, L, O, lane);
             else
-                put_partial(a, ((int64_t)c + h) * NC + j, O, M, L, lane);
+                put_partial(a, c, j, NC, O, M, L, lane);
         }
     }
 }
@@ -634,21 +636,21 @@ __device__ __forceinline__ void cta_tail(const DecodeArgs& a, unsigned char* rin
 #pragma unroll
             for (int o = 16; o >= 1; o >>= 1) L += __shfl_xor_sync(kFull, L, o);
         }
-        const int64_t sj = ((int64_t)c + h) * NC + j;
         if (!FUSED) {
+            const int64_t sj = ((int64_t)c + h) * NC + j;
             reinterpret_cast<float4*>(a.work_o + sj * kHeadDim)[lane] = O;
             if (lane == 0) *reinterpret_cast<float2*>(a.work_ml + sj * 2) = make_float2(M, L);
             continue;
         }
         if (after) {
-            put_partial(a, sj, O, M, L, lane);
+            put_partial(a, c, j, NC, O, M, L, lane);
             continue;
         }
         bool good = true;
         if (merger) {
             float* dep = reinterpret_cast<float*>(ring + warp * ring_bytes + dep_off);
             if (team == 1 || member > 0)
-                good = merge_partials<12, NCC>(a, h, j, NC, meta[TM::kC0] + max(member - 1, 0), team == 3 ? 2 : 1,
+                good = merge_partials<12, NCC>(a, j, NC, meta[TM::kC0] + max(member - 1, 0), team == 3 ? 2 : 1,
                                                    c + a.merge_extra, M, L, O, lane);
             if (member > 0) {
                 reinterpret_cast<float4*>(dep)[lane] = O;

@@ -97,7 +97,7 @@ struct DecodeArgs {
     float* work_ml;         // [slots][G][2]
     float* warp_o;          // [nparts][G][128]: a warp's state for a slab it left mid-range
     float* warp_ml;         // [nparts][G][2]
-    float* exch_o;          // fused-merge exchange: [slots][NC][128] and [slots][NC][2], every word 0 between launches
+    float* exch_o;          // fused-merge exchange: [CTAs][NC][128] and [CTAs][NC][2], every word 0 between launches
     float* exch_ml;
     float* out;             // [B][H][128]
     int32_t* slab_parts;    // [B*Hkv][2] tcgen05 kernel: first CTA and count of the CTAs that hold a part of the slab

@@ -71,3 +71,23 @@ def test_plans_made_and_released_by_several_threads():
         t.join()
     assert not errors, errors
     first.close()
+
+
+def test_memory_of_a_plan_of_many_slabs():
+    """What a plan of 512 sequences x 32 KV heads takes: the partials' workspace (one
+    record of 64 columns a CTA and a slab, one of 16 a warp), 16 columns a CTA for the
+    fused merge, and the metadata. Not a fused-merge slot a slab (136 MB)."""
+    import gc
+    B, Hkv = 512, 32
+    NH, rec = B * Hkv, 130 * 4
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sh = dkv.Shape(L=1, H=Hkv, H_kv=Hkv, D=1, bin_width=1)
+    gc.collect()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    plan = dkv.dkv_plan_dense(np.full(B, 3, np.int32), sh, 16)
+    torch.cuda.synchronize()
+    taken = free - torch.cuda.mem_get_info()[0]
+    plan.close()
+    bound = (sms + NH) * 64 * rec + sms * 16 * 16 * rec + sms * 16 * rec + 64 * NH
+    assert taken <= bound + (4 << 20)  # allocations come in pages of 2 MB
