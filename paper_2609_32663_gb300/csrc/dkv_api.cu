@@ -12,6 +12,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
 #include <map>
 #include <mutex>
 #include <new>
@@ -94,6 +95,18 @@ bool fault(const char* what)
 dkv_status cuda_fail(cudaError_t e, const char* where)
 {
     return fail(DKV_ERR_CUDA, "%s: %s", where, cudaGetErrorString(e));
+}
+
+// Runs f, which allocates host memory; a failure is reported, as no call throws.
+template <class F>
+dkv_status host_alloc(const char* what, F f)
+{
+    try {
+        f();
+    } catch (const std::exception&) {  // bad_alloc, or length_error for a size no vector has
+        return fail(DKV_ERR_OOM, "%s: host allocation failed", what);
+    }
+    return DKV_OK;
 }
 
 dkv_status dalloc(dkv::PlanMemory* m, size_t bytes, const char* what)
@@ -206,8 +219,11 @@ cudaError_t kernel_configs(int G, int B, int Hkv, KernelConfigs* out)
         (e = dkv::decode_config_mma(G, B, Hkv, 2, &k.multi)) != cudaSuccess ||
         (e = dkv::decode_config_tc(G, B, &k.tc)) != cudaSuccess)
         return e;
-    known.emplace(key, k);
     *out = k;
+    try {
+        known.emplace(key, k);
+    } catch (const std::bad_alloc&) {  // looked up again by the next plan
+    }
     return cudaSuccess;
 }
 
@@ -359,6 +375,14 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     // What the host gives: the counters' zeros, the pattern and the lengths, one copy.
     const ZeroBlock zb = take_zeroed(lay, p, 1);  // + the runs kernel's CTA counter
     const size_t o_M = lay.take<uint8_t>(nM), o_Tc = lay.take<int32_t>((size_t)B);
+    std::vector<uint8_t> given;
+    std::vector<int64_t> tail;
+    if ((st = host_alloc("copy of the pattern", [&] {
+             given.resize(lay.bytes - zb.off);
+             tail.resize((size_t)3 + s->L);
+             p->layer_rows.resize((size_t)s->L);
+         })) != DKV_OK)
+        return bail(st);
     if ((st = dalloc(&p->arena, lay.bytes, "plan metadata")) != DKV_OK)
         return bail(st);
     p->d_len = at<int32_t>(p->arena.ptr, o_len);
@@ -368,7 +392,6 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     place_zeroed(p, zb);
 
     cudaError_t e;
-    std::vector<uint8_t> given(lay.bytes - zb.off);
     if (nM) std::memcpy(given.data() + (o_M - zb.off), M_host, nM);
     std::memcpy(given.data() + (o_Tc - zb.off), ctx_len_host, (size_t)B * 4);
     if ((e = cudaMemcpyAsync(p->d_status, given.data(), given.size(), cudaMemcpyHostToDevice, stream)) != cudaSuccess)
@@ -401,14 +424,13 @@ static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len
     if ((st = launched(dkv::launch_map(ma, stream), "map kernels")) != DKV_OK) return bail(st);
     if ((st = plan_configs(p)) != DKV_OK) return bail(st);  // host work, while the kernels run
     // The one synchronisation: the totals (rows, kept rows, longest slab, rows of each layer).
-    std::vector<int64_t> tail((size_t)3 + s->L);
     if ((e = cudaMemcpyAsync(tail.data(), ma.tail, sizeof(int64_t) * tail.size(), cudaMemcpyDeviceToHost, stream)) !=
             cudaSuccess ||
         (e = cudaStreamSynchronize(stream)) != cudaSuccess)
         return bail(cuda_fail(e, "map: read totals"));
     p->total_rows = tail[0];
     p->kept_rows = tail[1];
-    p->layer_rows.assign(tail.begin() + 3, tail.end());
+    std::copy(tail.begin() + 3, tail.end(), p->layer_rows.begin());
     ArenaLayout lay2;
     const size_t o_idx = lay2.take<int32_t>((size_t)p->kept_rows), o_work = lay2.take<float>((size_t)p->work.total),
                  o_exch = lay2.take<float>((size_t)exch_floats(p));
@@ -477,8 +499,15 @@ dkv_status dkv_plan_dense(const int32_t* ctx_len_host, int32_t B, const dkv_shap
     // The uncompressed layout is given by the arguments: slab h holds the
     // sequence's Tc[b] rows at row h * T_stride.
     const int NH = s->L * B * s->H_kv;
-    std::vector<int32_t> len(NH);
-    std::vector<int64_t> off(NH + 1), ioff(NH + 1);
+    std::vector<int32_t> len;
+    std::vector<int64_t> off, ioff;
+    if ((st = host_alloc("dense plan metadata", [&] {
+             len.resize((size_t)NH);
+             off.resize((size_t)NH + 1);
+             ioff.resize((size_t)NH + 1);
+             p->layer_rows.assign((size_t)s->L, 0);
+         })) != DKV_OK)
+        return bail(st);
     int64_t run = 0;
     for (int h = 0; h < NH; ++h) {
         const int b = (h / s->H_kv) % B;
@@ -491,7 +520,6 @@ dkv_status dkv_plan_dense(const int32_t* ctx_len_host, int32_t B, const dkv_shap
     ioff[NH] = run;
     p->total_rows = off[NH];
     p->kept_rows = run;
-    p->layer_rows.assign((size_t)s->L, 0);
     for (int h = 0; h < NH; ++h) p->layer_rows[(size_t)h / (B * s->H_kv)] += len[h];
     ArenaLayout lay;
     const size_t o_len = lay.take<int32_t>((size_t)NH), o_off = lay.take<int64_t>((size_t)NH + 1),
@@ -589,11 +617,16 @@ dkv_status dkv_vmm_trim(dkv_vmm* m, const dkv_plan* p, int32_t guard_rows, int64
     if (dkv::vmm_bytes(m) < need)
         return fail(DKV_ERR_INVALID_ARG, "buffer of %lld bytes is smaller than the plan's cache (%lld bytes)",
                     (long long)dkv::vmm_bytes(m), (long long)need);
-    std::vector<int32_t> len((size_t)NH);
+    const int64_t page = dkv::vmm_page(m), npages = dkv::vmm_bytes(m) / page;
+    std::vector<int32_t> len;
+    std::vector<uint8_t> keep;
+    const dkv_status st = host_alloc("lengths and pages", [&] {
+        len.resize((size_t)NH);
+        keep.resize((size_t)npages);
+    });
+    if (st != DKV_OK) return st;
     cudaError_t e = cudaMemcpy(len.data(), p->d_len, sizeof(int32_t) * NH, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "read lengths");
-    const int64_t page = dkv::vmm_page(m), npages = dkv::vmm_bytes(m) / page;
-    std::vector<uint8_t> keep((size_t)npages);
     dkv::vmm_pages_to_keep(len.data(), NH, p->inplace_stride, p->reserve, guard_rows, dkv::kRowBytes, page, npages,
                            keep.data());
     return dkv::vmm_release_pages(m, keep.data(), npages, freed_bytes);

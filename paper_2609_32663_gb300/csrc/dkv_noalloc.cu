@@ -22,6 +22,7 @@
 #include <cstdio>
 #include <map>
 #include <mutex>
+#include <new>
 #include <tuple>
 #include <vector>
 
@@ -59,17 +60,25 @@ cudaError_t setup_for_current_context(int G, int B, void** scratch, dkv::DecodeC
     if (!addr) {
         e = cudaGetSymbolAddress(&addr, g_decode_scratch);
         if (e != cudaSuccess) return e;
-        g_scratch_addr.emplace_back(id, addr);
+        try {
+            g_scratch_addr.emplace_back(id, addr);
+        } catch (const std::bad_alloc&) {  // looked up again by the next call
+        }
     }
     const auto key = std::make_tuple(id, G, B);
     auto it = g_configs.find(key);
     if (it == g_configs.end()) {
         dkv::DecodeConfig c{};
         if ((e = dkv::decode_config(G, B, &c)) != cudaSuccess) return e;
-        it = g_configs.emplace(key, c).first;
+        *cfg = c;
+        try {
+            g_configs.emplace(key, c);
+        } catch (const std::bad_alloc&) {  // looked up again by the next call
+        }
+    } else {
+        *cfg = it->second;
     }
     *scratch = addr;
-    *cfg = it->second;
     return cudaSuccess;
 }
 

@@ -13,6 +13,7 @@
 #include <cuda.h>
 
 #include <mutex>
+#include <new>
 #include <vector>
 
 namespace dkv {
@@ -66,13 +67,17 @@ cudaError_t current_context_id(unsigned long long* id)
 
 namespace {
 
-// The entry of context `id`; g_mu is held.
-Context& context_of(unsigned long long id)
+// The entry of context `id`, null if the host has no memory for one; g_mu is held.
+Context* context_of(unsigned long long id)
 {
     for (Context& c : g_contexts)
-        if (c.id == id) return c;
-    g_contexts.push_back(Context{id, 0, 0, {}});
-    return g_contexts.back();
+        if (c.id == id) return &c;
+    try {
+        g_contexts.push_back(Context{id, 0, 0, {}});
+    } catch (const std::bad_alloc&) {
+        return nullptr;
+    }
+    return &g_contexts.back();
 }
 
 void give_back(Context& c)
@@ -91,7 +96,9 @@ cudaError_t plan_alloc(PlanMemory* m, size_t bytes)
     cudaError_t e = current_context_id(&id);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(g_mu);
-    Context& c = context_of(id);
+    Context* entry = context_of(id);
+    if (!entry) return cudaErrorMemoryAllocation;
+    Context& c = *entry;
     // The smallest kept block that fits, unless it is more than twice as large.
     size_t best = c.kept.size();
     for (size_t i = 0; i < c.kept.size(); ++i)
@@ -126,14 +133,16 @@ void plan_free(const PlanMemory& m, bool idle)
     unsigned long long id = 0;
     const bool own = current_context_id(&id) == cudaSuccess && id == m.context;
     std::lock_guard<std::mutex> lock(g_mu);
-    Context& c = context_of(m.context);
+    Context& c = *context_of(m.context);  // (there since plan_alloc)
     --c.live;
-    if (own && idle && c.live > 0 && c.kept_bytes + m.bytes <= kKeepBytes) {
-        c.kept.push_back(m);
-        c.kept_bytes += m.bytes;
-    } else {
-        cudaFree(m.ptr);
-    }
+    bool keep = own && idle && c.live > 0 && c.kept_bytes + m.bytes <= kKeepBytes;
+    if (keep) try {
+            c.kept.push_back(m);
+            c.kept_bytes += m.bytes;
+        } catch (const std::bad_alloc&) {
+            keep = false;
+        }
+    if (!keep) cudaFree(m.ptr);
     if (own && c.live == 0) give_back(c);
 }
 

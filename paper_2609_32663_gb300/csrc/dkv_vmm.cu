@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <cstdio>
+#include <exception>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -140,11 +141,16 @@ dkv_status dkv_vmm_alloc(int64_t bytes, dkv_vmm** out, void** dptr)
     m->bytes = (bytes + m->page - 1) / m->page * m->page;
     m->device = device;
     const int64_t npages = m->bytes / m->page;
+    try {
+        m->handles.assign((size_t)npages, 0);
+    } catch (const std::exception&) {
+        delete m;
+        return fail(DKV_ERR_OOM, "host allocation for %lld pages failed", npages);
+    }
     if (v.reserve(&m->base, m->bytes, m->page, 0, 0) != CUDA_SUCCESS) {
         delete m;
         return fail(DKV_ERR_OOM, "cuMemAddressReserve of %lld bytes failed", bytes);
     }
-    m->handles.assign((size_t)npages, 0);
     for (int64_t i = 0; i < npages; ++i) {
         CUmemGenericAllocationHandle h = 0;
         if (v.create(&h, m->page, &prop, 0) != CUDA_SUCCESS) {
