@@ -168,3 +168,26 @@ def test_outputs_of_a_timed_out_multi_query_call_stay_unwritten(monkeypatch, Hkv
     assert torch.equal(again, first)
     assert dkv.dkv_plan_status(c.plan) == 0
     c.close()
+
+
+@pytest.mark.parametrize("Q", [1, 2, 4, 5, 16])
+def test_values_of_plans_of_other_sizes_side_by_side(Q):
+    """Every multi-query kernel of a large plan after plans of fewer sequences and KV
+    heads were made: with q = 0 an output is the mean of its slab's V rows."""
+    big = Case(wl(H=4 * 16, Hkv=16, T=1300, B=20), reserve=2)
+    small = [Case(wl(H=4 * h, Hkv=h, T=1300, B=b), reserve=2) for h, b in ((1, 1), (8, 1), (2, 3))]
+    for c in [big] + small:
+        B, H, Hkv = c.wl.B, c.wl.H, c.wl.Hkv
+        out = torch.full((B, Q, H, 128), float("nan"), device=c.dev)
+        q = torch.zeros(out.shape, dtype=torch.bfloat16, device=c.dev)
+        dkv.dkv_decode_multi(c.plan, 0, q, Q, None, c.Kc, c.Vc, out)
+        off = c.om.off[:-1].reshape(B, Hkv)
+        ln = c.om.len.reshape(B, Hkv)
+        for b in range(B):
+            for g in range(Hkv):
+                mean = c.Vc[int(off[b, g]):int(off[b, g] + ln[b, g])].double().mean(dim=0)
+                got = out[b, :, 4 * g:4 * g + 4].double()
+                assert (got - mean).abs().max().item() <= 1e-5
+        assert dkv.dkv_plan_status(c.plan) == 0
+    for c in [big] + small:
+        c.close()
