@@ -104,8 +104,9 @@ const char* dkv_last_error(void);
  * list and the caller's packed caches). The index list is then written by a
  * kernel that the call leaves running on `stream`: work queued on `stream`
  * afterwards is ordered after it; other streams must wait for `stream`.
- * Device memory: one allocation for the plan's metadata and counters, and one,
- * sized after the sync, for the index list and the split-K workspace.
+ * Device memory: one block for the plan's metadata and counters, and one, sized
+ * after the sync, for the index list, the split-K workspace and the fused merge's
+ * exchange. A block of a released plan may serve (see dkv_free).
  */
 dkv_status dkv_map_pattern(const uint8_t* M_host, const int32_t* ctx_len_host, int32_t B,
                            const dkv_shape* s, int32_t reserve_rows, cudaStream_t stream,
@@ -274,7 +275,8 @@ dkv_status dkv_decode_attn(const dkv_plan* plan, int32_t layer, const void* q,
  * (num_queries * G of them) share every K/V row, so the rows are read once for
  * all queries:
  *   <= 16 columns  a split-K kernel whose warps multiply 16-row tiles on the
- *                  warp-level tensor-core path, then a combine kernel;
+ *                  warp-level tensor-core path, with the merge of the slabs that
+ *                  several CTAs share fused in;
  *   17..64         a tcgen05 kernel: 64-row tiles staged by TMA, scores and
  *                  outputs accumulated in tensor memory; then a combine kernel
  *                  merges the slabs that several CTAs share.
@@ -349,7 +351,13 @@ dkv_status dkv_decode_attn_noalloc(const dkv_shape* s, int32_t B, int32_t layer,
                                    const int32_t* n_appended, void* Kc, void* Vc, float scale,
                                    float* out, int32_t* status, cudaStream_t stream);
 
-/* Release a plan (NULL-safe). Synchronises the device before freeing. */
+/*
+ * Release a plan (NULL-safe). Synchronises the plan's device first. While other plans
+ * of the same CUDA context are alive, its device memory is kept for the next plan made
+ * there (at most 64 MB a context; not if the synchronisation failed or another context
+ * is current); the release of a context's last plan, made while that context is
+ * current, gives all of it back, and so does an allocation that does not fit otherwise.
+ */
 void dkv_free(dkv_plan* plan);
 
 /*

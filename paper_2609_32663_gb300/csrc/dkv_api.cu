@@ -256,8 +256,8 @@ dkv_status plan_configs(dkv_plan* p)
 // Floats of the fused merge's exchange.
 int64_t exch_floats(const dkv_plan* p) { return p->exch_slots * dkv::kMaxCols * (dkv::kHeadDim + 2); }
 
-// Places the counters (status word, then the fused combine's slab counters) as
-// one int32 block that a single memset zeroes, and the split-K workspace.
+// Places what starts as zeros: the status word (and a pad), the slab_parts words of the
+// tcgen05 kernel, and `extra` counters, one int32 block.
 struct ZeroBlock {
     size_t off = 0, count = 0;
 };
@@ -307,13 +307,13 @@ const char* dkv_last_error(void) { return g_err; }
 // The map of dkv_map_pattern and dkv_map_pattern_inplace: slab offsets are the
 // running sum of (len + reserve), or h * inplace_stride when that is > 0.
 //
-// Device work, all on `stream`: one allocation for the plan's metadata and
-// counters (the map's inputs M and Tc live there too), one memset of the
-// counters, the copies of M and Tc, the runs kernel (and, in place, the slab
+// Device work, all on `stream`: a block of memory for the plan's metadata and
+// counters (the map's inputs M and Tc live there too), one copy of what the host
+// gives (the counters' zeros, M and Tc), the runs kernel (and, in place, the slab
 // order), one read of the totals -- the only synchronisation -- then a second
-// allocation, sized by the totals, for the index list and the split-K
-// workspace, and the index list's write. The call returns without waiting for
-// the write: later calls on `stream` are ordered after it.
+// block, sized by the totals, for the index list, the split-K workspace and the
+// exchange, a memset of the exchange, and the index list's write. The call returns
+// without waiting for the write: later calls on `stream` are ordered after it.
 static dkv_status map_pattern_impl(const uint8_t* M_host, const int32_t* ctx_len_host, int32_t B,
                                    const dkv_shape* s, int32_t reserve_rows, int64_t inplace_stride,
                                    cudaStream_t stream, dkv_plan** out)
@@ -667,9 +667,11 @@ namespace {
 // CTAs of a tensor-core launch over one layer: half the grid for a layer of
 // fewer than kSmallLaunchRows kept rows. Half the SMs already draw the full HBM
 // bandwidth, and a layer of 26 MB streams in a few microseconds, so fewer
-// partials per slab (a shorter end-of-pass merge) count for more there:
-// measured 3.5 % faster per step at a 16K context, equal at 128K, 1 % slower
-// at 32K (50 MB layers), hence the bound.
+// partials per slab (a shorter end-of-pass merge) count for more there. us per step
+// with half and with all CTAs, by kept rows a layer: G = 4, 18K rows 275 / 297, 32K
+// rows 293 / 319, 52K rows 336 / 361, 79K rows 406 / 397, 89K rows 467 / 431; G = 7, 8K
+// rows 298 / 351, 25K rows 332 / 367, 47K rows 365 / 413, 76K rows 418 / 434; G = 2
+// within 2 % up to 52K rows, 79K rows 399 / 369. Hence the bound.
 constexpr int64_t kSmallLaunchRows = 65536;  // 32 MB of K and V rows
 int launch_ctas(const dkv_plan* p, int layer, const dkv::DecodeConfig& cfg)
 {

@@ -25,9 +25,11 @@
 // the previous kernel ends, and the merge after the last row. The work of those
 // parts is scalar and runs once, so it is kept short: warp-uniform values are
 // marked as such (without that every vote and shuffle carries a check for a
-// split warp), rare code is out of line (79 -> 55 KB), nothing lives in a stack
-// frame. Same-box us per step, 32 layers: 128K 1,065 -> 1,017, 32K 469 -> 422,
-// 4K 312 -> 259; Qwen shape 64K x 4, 28 layers: 982 -> 919.
+// split warp), rare code is out of line, nothing lives in a stack frame. Same-box
+// us per step, 32 layers: 128K 1,065 -> 1,017, 32K 469 -> 422, 4K 312 -> 259; Qwen
+// shape 64K x 4, 28 layers: 982 -> 919. (Rows appended by earlier calls, which are
+// fetched only after the previous kernel, then cost 0.5 % at 128K and 1 % at 32K, with
+// half of a reserve of 256 filled.)
 #include "dkv_decode_common.cuh"
 
 #include <cuda.h>

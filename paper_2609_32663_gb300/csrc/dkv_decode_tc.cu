@@ -63,11 +63,12 @@
 //
 // What bounds it: a 64-row tile is 32 KB, 0.73 us at an SM's share of HBM, and its
 // products need 0.3 us of the tensor pipe's operand bandwidth, so the schedules of
-// the roles set the pace. They run on warp-uniform values (uniform()): with a
-// single-lane MMA loop every operand went through a vector register and a move
-// before each product, and the kernel's code was 136 KB of walkers and partition
-// arithmetic, repeated inline, now 75. Same box, 4 layers at 128K: 64 columns 236
-// -> 189 us, 32 columns 229 -> 173; Qwen shape 64K x 4, 28 columns 250 -> 180.
+// the roles set the pace. The TMA and MMA roles run whole warps on warp-uniform values
+// (uniform()) and one lane issues, where a single lane ran the loop; the walkers and the
+// partition are out of line, once a CTA, where every role had its own inline. Same box,
+// 4 layers at 128K: 64 columns 236 -> 189 us, 32 columns 229 -> 173; Qwen shape 64K x 4,
+// 28 columns 250 -> 180. (With the second launch and without the boxes past a segment:
+// 64 columns 170, 28 columns 154.)
 #include "dkv_decode_common.cuh"
 
 #include <cuda.h>
@@ -505,8 +506,7 @@ __device__ __forceinline__ TcPart tc_partition(const DecodeArgs& a, const SeqTab
     return part;
 }
 
-// One warp computes the CTA's share (A = Bc: no rows). Out of line and once: with
-// this inlined wherever it was needed the kernel's code was 136 KB.
+// One warp computes the CTA's share (A = Bc: no rows), once and out of line.
 __device__ __noinline__ void tc_share(const DecodeArgs& a, unsigned char* table, int c, TcShare* out)
 {
     const SeqTable tab = seq_table_at(table, a);
@@ -746,10 +746,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         // score product needs its K stage, its S buffer free (the output product
         // of tile t - 4 issued, so its softmax is done) and, first in a segment,
         // the segment's Q; an output product needs its P and its V stage. The whole
-        // warp runs the schedule on warp-uniform values and one lane issues: the
-        // products' operands are then uniform registers, which is what tcgen05.mma
-        // takes (a single-lane loop moved each of them there before each product:
-        // ~100 cycles a product instead of the pipe's 46 to 64).
+        // warp runs the schedule on warp-uniform values and one lane issues (a
+        // single-lane loop took ~100 cycles a product instead of the pipe's 46 to 64).
         {
             const bool leads = elect_one();
             const uint32_t id1 = idesc(kTcQRows, kTcRows, 0, 0);

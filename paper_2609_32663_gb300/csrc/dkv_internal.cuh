@@ -113,8 +113,8 @@ struct DecodeArgs {
     int merge_extra;        // partials a fused merge waits for beyond the other CTAs' (0; 1 injects a wait that runs out)
 };
 
-// Most columns (queries x group heads) one decode call handles; the plan's
-// split-K workspace and arrival counters are sized for this many.
+// Most columns (queries x group heads) a call of the mma.sync and fp32 kernels
+// handles; the plan's warp records and exchange are sized for this many.
 constexpr int kMaxCols = 16;
 // Most columns of one tcgen05 multi-query call (its CTA partials are sized for this many).
 constexpr int kTcMaxCols = 64;
